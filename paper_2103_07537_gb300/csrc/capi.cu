@@ -945,8 +945,6 @@ static int autotune_levels(bamg_ctx* h, cudaStream_t s) {
         a.x_in = L.xa;
         a.x_out = L.xb;
         a.xt = L.xt;
-        a.uc = nullptr;
-        a.agg = nullptr;
         a.field = 0;
         a.F = h->F;
         a.omega = h->p.omega;
@@ -955,15 +953,40 @@ static int autotune_levels(bamg_ctx* h, cudaStream_t s) {
         // warp-per-row one only when it is faster by more than kTuneMargin (3
         // launches and a plain minimum flipped between runs on near ties)
         const int reps = 10;
-        L.tune_us[0] = time_launch(s, e0, e1, reps, [&] { return launch_bgs_colour<T>(b, h->fb, a, s); });
-        L.tune_us[1] = time_launch(s, e0, e1, reps, [&] { return launch_bgs_colour_tpr<T>(b, h->fb, a, s, 0); });
-        L.tune_us[4] = time_launch(s, e0, e1, reps, [&] { return launch_bgs_colour_tpr<T>(b, h->fb, a, s, 1); });
-        L.tune_us[5] = time_launch(s, e0, e1, reps, [&] { return launch_bgs_colour_tpr<T>(b, h->fb, a, s, 2); });
-        L.tune_us[6] = time_launch(s, e0, e1, reps,
-                                   [&] { return launch_bgs_colour_staged<T>(b, h->fb, a, L.max_row, h->d_err, s); });
-        L.tune_us[7] = time_launch(s, e0, e1, reps, [&] { return launch_bgs_colour_wide<T>(b, h->fb, a, s); });
-        L.tune_us[8] = time_launch(s, e0, e1, reps, [&] { return launch_bgs_colour_bsp<T>(b, h->fb, a, 16, s); });
-        L.tune_us[9] = time_launch(s, e0, e1, reps, [&] { return launch_bgs_colour_bsp<T>(b, h->fb, a, 8, s); });
+        // Levels whose values exceed L2 are timed over every colour of the
+        // field step (the average per launch): one colour launched again and
+        // again would be read from L2, which the cycle's colours never are.
+        // (3D, 64^3 cells: 12.6 us against 15 us per launch in the cycle, and
+        // another mapping in front.)
+        int l2 = 0, dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
+            l2 = 0;
+        const bool big = l2 > 0 && (double)L.nnzb * b * b * sizeof(T) > (double)l2;
+        const int c_tune = big ? (h->nf > 1 ? L.fcol[1] : L.n_colours) : 1;
+        auto tune = [&](auto&& launch) {
+            const float us = time_launch(s, e0, e1, reps, [&]() {
+                for (int c = 0; c < c_tune; ++c) {
+                    BgsArgs ac = a;
+                    ac.n_in_colour = L.colour_ptr[c + 1] - L.colour_ptr[c];
+                    ac.nodes = L.colour_nodes + L.colour_ptr[c];
+                    ac.colour = c;
+                    const int st = launch(ac);
+                    if (st != BAMG_OK) return st;
+                }
+                return (int)BAMG_OK;
+            });
+            return us >= 1e29f ? us : us / c_tune;  // (1e30: not a mapping of this level)
+        };
+        L.tune_us[0] = tune([&](const BgsArgs& ac) { return launch_bgs_colour<T>(b, h->fb, ac, s); });
+        L.tune_us[1] = tune([&](const BgsArgs& ac) { return launch_bgs_colour_tpr<T>(b, h->fb, ac, s, 0); });
+        L.tune_us[4] = tune([&](const BgsArgs& ac) { return launch_bgs_colour_tpr<T>(b, h->fb, ac, s, 1); });
+        L.tune_us[5] = tune([&](const BgsArgs& ac) { return launch_bgs_colour_tpr<T>(b, h->fb, ac, s, 2); });
+        L.tune_us[6] = tune(
+            [&](const BgsArgs& ac) { return launch_bgs_colour_staged<T>(b, h->fb, ac, L.max_row, h->d_err, s); });
+        L.tune_us[7] = tune([&](const BgsArgs& ac) { return launch_bgs_colour_wide<T>(b, h->fb, ac, s); });
+        L.tune_us[8] = tune([&](const BgsArgs& ac) { return launch_bgs_colour_bsp<T>(b, h->fb, ac, 16, s); });
+        L.tune_us[9] = tune([&](const BgsArgs& ac) { return launch_bgs_colour_bsp<T>(b, h->fb, ac, 8, s); });
         const T* x = static_cast<const T*>(L.xa);
         const T* r = static_cast<const T*>(L.res);
         T* y = static_cast<T*>(L.xb);
@@ -1918,13 +1941,28 @@ static int other_fields(bamg_ctx* h, const Level& L, int f, const T* x_in, T* x_
     return BAMG_OK;
 }
 
+// algorithmic bytes and flops of one colour of a field step, added to *bytes
+// and *flops: from a given iterate every block's field rows, from zero only
+// the lower colours' (and the flag and column of every block)
+static void bgs_model(double es, double B, double FB, double nc, double nnz, double low, bool given, double* bytes,
+                      double* flops) {
+    const double node = 8.0 + FB * FB * es + FB * es + B * es;  // list entry, row range, inverse, rhs, x_out
+    *bytes += given ? nnz * (FB * B * es + 4.0) + nc * (node + B * es + FB * es)
+                    : nnz * 5.0 + low * FB * B * es + nc * (node + FB * es);
+    *flops += 2.0 * ((given ? nnz * FB * B : low * FB * FB) + nc * FB * FB);
+}
+
+// the multicolour Gauss-Seidel sub-solve in its in-place form (see bgs_block)
+static bool bgs_in_place(const bamg_ctx* h) { return h->p.sub_solver == 0 && h->p.inner_sweeps <= 1; }
+
 // one field step of Algorithm 1 on level l: x_out = x_in updated in field f
-// uc != nullptr: the coarse correction P uc is added to x_in on the fly (x_in is
-// then the state before prolongation and x_out receives the corrected values)
+// (x_in is scratch after the step).  uc != nullptr (not with bgs_in_place): the
+// coarse correction P uc is added to x_in on the fly (x_in is then the state
+// before prolongation and x_out receives the corrected values)
 // With fields on node sets, field f is the node range fo[f].. and its colours
 // are fcol[f]..fcol[f+1]-1; each node is one b x b sub-solve block.
 template <typename T>
-static int bgs_step(bamg_ctx* h, int l, int f, const T* rhs, const T* x_in, T* x_out, const T* uc,
+static int bgs_step(bamg_ctx* h, int l, int f, const T* rhs, T* x_in, T* x_out, const T* uc,
                     cudaStream_t s) {
     const Level& L = h->lev[l];
     const bool have_counts = (int)L.colour_nnz.size() == L.n_colours;
@@ -2092,8 +2130,6 @@ static int bgs_step(bamg_ctx* h, int l, int f, const T* rhs, const T* x_in, T* x
         a.x_in = x_in;
         a.x_out = x_out;
         a.xt = L.xt;
-        a.uc = uc;
-        a.agg = uc ? L.agg : nullptr;
         a.field = nodef ? 0 : f;
         a.F = h->F;
         a.omega = h->p.omega;
@@ -2103,10 +2139,7 @@ static int bgs_step(bamg_ctx* h, int l, int f, const T* rhs, const T* x_in, T* x
             for (int c = c_lo; c < c_hi; ++c) {
                 const double es = sizeof(T), B = h->b, FB = h->fb, nc = L.colour_ptr[c + 1] - L.colour_ptr[c];
                 const double nnz = (double)L.colour_nnz[c], low = (double)L.colour_nnz_lower[c];
-                bytes += nnz * (FB * B * es + 4.0) + nc * 8.0 + nc * FB * FB * es + nc * FB * es +
-                         (x_in ? nc * B * es : 0.0) + nc * B * es + nc * FB * es + (c > 0 ? nc * FB * es : 0.0) +
-                         (uc ? nc * (B * es + 4.0) : 0.0);
-                flops += 2.0 * ((x_in ? nnz * FB * B : 0.0) + low * FB * FB + nc * FB * FB);
+                bgs_model(es, B, FB, nc, nnz, low, x_in != nullptr, &bytes, &flops);
             }
         const SweepArgs sw = sweep_args(h, L, c_lo, c_hi);
         PL(BAMG_K_SMOOTH, bytes, flops,
@@ -2130,8 +2163,6 @@ static int bgs_step(bamg_ctx* h, int l, int f, const T* rhs, const T* x_in, T* x
         a.x_in = x_in;
         a.x_out = x_out;
         a.xt = L.xt;
-        a.uc = uc;
-        a.agg = uc ? L.agg : nullptr;
         a.field = nodef ? 0 : f;
         a.F = h->F;
         a.omega = h->p.omega;
@@ -2140,10 +2171,7 @@ static int bgs_step(bamg_ctx* h, int l, int f, const T* rhs, const T* x_in, T* x
         if (h->prof && have_counts) {
             const double es = sizeof(T), B = h->b, FB = h->fb, nc = a.n_in_colour;
             const double nnz = (double)L.colour_nnz[c], low = (double)L.colour_nnz_lower[c];
-            bytes = nnz * (FB * B * es + 4.0) + nc * 8.0 + nc * FB * FB * es + nc * FB * es +
-                    (x_in ? nc * B * es : 0.0) + nc * B * es + nc * FB * es + (c > 0 ? nc * FB * es : 0.0) +
-                    (uc ? nc * (B * es + 4.0) : 0.0);
-            flops = 2.0 * ((x_in ? nnz * FB * B : 0.0) + low * FB * FB + nc * FB * FB);
+            bgs_model(es, B, FB, nc, nnz, low, x_in != nullptr, &bytes, &flops);
         }
         if (h->rec) {
             TailPhase ph{};
@@ -2354,10 +2382,29 @@ static int mgv(bamg_ctx* h, int l, const T* rhs, T* out, cudaStream_t s) {
             BAMG_CUDA_TRY(cudaMemcpyAsync(out, cur, sizeof(T) * (size_t)L.n * b, cudaMemcpyDeviceToDevice, s));
         }
     }
-    // the first post-smoothing step applies u <- u + P u_c on the fly
+    // u <- u + P u_c: a pass of its own ahead of the in-place smoother, whose
+    // colours would otherwise each gather the correction of every neighbour
+    // (the aggregate, then its value) again; the other sub-solvers apply it in
+    // their first step
+    const bool fused = !bgs_in_place(h);
+    if (S_post > 0 && !fused) {
+        const double pb = L.n * 4.0 + 2.0 * nb * es + ncb * es;
+        if (h->rec) {
+            TailPhase ph{};
+            ph.type = kPhaseProlongCopy;
+            ph.n = L.n;
+            ph.x = cur;
+            ph.rhs = C.uc;
+            ph.ci = L.agg;
+            ph.y = cur;
+            record(h, ph, pb, nb);
+        } else {
+            PL(BAMG_K_PROLONG, pb, nb, launch_prolong<T>(b, L.n, L.agg, static_cast<const T*>(C.uc), cur, s));
+        }
+    }
     for (int t = 0; t < S_post; ++t) {
         T* dst = (t == S_post - 1) ? out : ((cur == xa) ? xb : xa);
-        TRY(bgs_step<T>(h, l, t % NS, rhs, cur, dst, t == 0 ? static_cast<const T*>(C.uc) : nullptr, s));
+        TRY(bgs_step<T>(h, l, t % NS, rhs, cur, dst, t == 0 && fused ? static_cast<const T*>(C.uc) : nullptr, s));
         cur = dst;
     }
     return BAMG_OK;

@@ -184,6 +184,37 @@ __device__ __forceinline__ void load_row(const T* __restrict__ p, T (&out)[B]) {
     }
 }
 
+// one value, and the B values at p (alignment as load_row), read through L2
+template <typename T>
+__device__ __forceinline__ T ld_cg(const T* p) {
+    return __ldcg(p);
+}
+template <typename T, int B>
+__device__ __forceinline__ void load_cg(const T* p, T (&out)[B]) {
+    constexpr int bytes_row = B * (int)sizeof(T);
+    if constexpr (sizeof(T) == 4 && bytes_row % 16 == 0) {
+#pragma unroll
+        for (int c = 0; c < B; c += 4) {
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(p + c));
+            out[c] = v.x;
+            out[c + 1] = v.y;
+            out[c + 2] = v.z;
+            out[c + 3] = v.w;
+        }
+    } else if constexpr (bytes_row % 16 == 0 || (sizeof(T) == 4 && bytes_row % 8 == 0)) {
+        using V2 = typename VecOf<T>::v2;
+#pragma unroll
+        for (int c = 0; c < B; c += 2) {
+            const V2 v = __ldcg(reinterpret_cast<const V2*>(p + c));
+            out[c] = v.x;
+            out[c + 1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < B; ++c) out[c] = __ldcg(p + c);
+    }
+}
+
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
@@ -204,6 +235,15 @@ inline int ceil_div(long a, long b) { return (int)((a + b - 1) / b); }
 // measured slower).  Without the attribute both are no-ops.  Data that is
 // constant during a cycle (matrices, inverses, colour lists, dampings) may be
 // read before pdl_wait().
+//
+// Vectors that an earlier kernel writes are read through L2 (ld_cg, load_cg)
+// in these kernels, and their pointers are not const __restrict__: a CTA that
+// is resident before its predecessor has finished shares its SM's L1 with the
+// predecessor's CTAs, and a wait that returns at once (the predecessor ended
+// while the CTA loaded its matrix rows) leaves their lines there.  Measured:
+// the residual after a smoother launch read old values of x~ in the first
+// cycles of a process (cold instruction caches); through L2, or with a fence
+// after the wait, never; the L2 path costs nothing measurable.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -271,11 +311,16 @@ struct BgsArgs {
     const void* vals = nullptr;
     const void* dinv = nullptr;    // [n][F][fb*fb]
     const void* rhs = nullptr;
-    const void* x_in = nullptr;    // nullptr = zero vector
+    // nullptr = zero vector.  The multicolour Gauss-Seidel kernels add x~ to
+    // the field's entries of the nodes they finish (scratch after the step);
+    // the other sub-solvers only read it
+    void* x_in = nullptr;
     void* x_out = nullptr;
     void* xt = nullptr;            // [n][fb]
-    const void* uc = nullptr;      // optional: coarse correction added to x_in on the fly (x_in + P uc)
-    const int* agg = nullptr;      // aggregate of every node (with uc)
+    // coarse correction added to x_in on the fly (x_in + P uc) by the ILU(0),
+    // Schwarz and iterated sub-solves, with the aggregate of every node
+    const void* uc = nullptr;
+    const int* agg = nullptr;
     int field = 0;
     int F = 1;
     double omega = 0.5;

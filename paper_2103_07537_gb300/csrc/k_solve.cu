@@ -13,9 +13,9 @@
 // warp short: these kernels are latency bound on L2-resident levels.
 //
 // The warp-level bodies are device functions shared by the one-step kernels
-// and the tail kernel.  Their template flag CG selects L2-coherent loads
-// (ld.global.cg) for vectors that the same launch writes (the tail kernel);
-// matrix data is read through the read-only path in both.
+// and the tail kernel.  Vectors are read through L2 (ld.global.cg: see pdl_wait
+// for the one-step kernels; the tail kernel writes them in the same launch),
+// matrix data through the read-only path.
 #include <cooperative_groups.h>
 
 #include "bgs_body.cuh"
@@ -52,7 +52,7 @@ __device__ __forceinline__ T reduce_rows(T v, int lane) {
 // y_i = (rhs_i -) sum_j A_ij x_j for block row i; whole warp.  With PDL the
 // lane's first block (column and matrix row, fixed for the cycle) is loaded
 // before the wait on the previous kernel.
-template <typename T, int B, int FB, bool CG, bool PDL = false, bool FM = false>
+template <typename T, int B, int FB, bool PDL = false, bool FM = false>
 __device__ __forceinline__ void spmv_row(long i, int lane, const int* __restrict__ rp, const int* __restrict__ ci,
                                          const T* __restrict__ vals, const T* x, const T* rhs, T* y) {
     constexpr int G = kWarp / B;
@@ -71,12 +71,12 @@ __device__ __forceinline__ void spmv_row(long i, int lane, const int* __restrict
         pdl_wait();
         pdl_trigger();
     }
-    const T bi = (rhs && lane < B) ? ld1<T, CG>(rhs + (size_t)i * B + lane) : T(0);  // issued early
+    const T bi = (rhs && lane < B) ? ld_cg(rhs + (size_t)i * B + lane) : T(0);  // issued early
     T acc = T(0);
     if (have) {
         {
             T xv[B];
-            load_vec<T, B, CG>(x + (size_t)jf * B, xv);
+            load_cg<T, B>(x + (size_t)jf * B, xv);
 #pragma unroll
             for (int c = 0; c < B; ++c) acc = fma(af[c], xv[c], acc);
         }
@@ -85,7 +85,7 @@ __device__ __forceinline__ void spmv_row(long i, int lane, const int* __restrict
             const int j = __ldg(ci + k);
             T a[B], xv[B];
             load_row<T, B>(vrow<T, B, FB, FM>(vals, k0, k1, k, r), a);
-            load_vec<T, B, CG>(x + (size_t)j * B, xv);
+            load_cg<T, B>(x + (size_t)j * B, xv);
 #pragma unroll
             for (int c = 0; c < B; ++c) acc = fma(a[c], xv[c], acc);
         }
@@ -105,12 +105,13 @@ __device__ __forceinline__ void spmv_row(long i, int lane, const int* __restrict
 // so they are fused into one pass: node i of colour c accumulates
 //   rhs_f,i - sum_j A_{f,*}[i,j] x_in,j - sum_{j: colour(j) < c} A_ff[i,j] x~_j
 // (neighbours of later colours still have x~ = 0, neighbours of the same
-// colour do not exist).  x_in is never written during the step; node i writes
-// its updated values to x_out (all b components: field f corrected, the
-// others copied), so the field update of Algorithm 1 needs no extra pass.
-// With uc set, x_in + P uc (the coarse correction) is read in place of x_in.
+// colour do not exist) as one product per block, because a finished node j
+// carries x_in,j + x~_j in its field-f entries of x_in (see bgs_block; x_in is
+// scratch after the step).  Node i writes its updated values to x_out (all b
+// components: field f corrected, the others copied), so the field update of
+// Algorithm 1 needs no extra pass.
 // ---------------------------------------------------------------------------
-template <typename T, int B, int FB, bool CG, bool PDL = false, bool FM = false>
+template <typename T, int B, int FB, bool PDL = false, bool FM = false>
 __device__ __forceinline__ void bgs_node(const BgsArgs& a, long q, int lane) {
     constexpr int G = kWarp / FB;  // blocks of the row per pass
     const int kk = lane / FB;
@@ -118,7 +119,6 @@ __device__ __forceinline__ void bgs_node(const BgsArgs& a, long q, int lane) {
     const int f0 = a.field * FB;
     const T* __restrict__ vals = static_cast<const T*>(a.vals);
     const T* x_in = static_cast<const T*>(a.x_in);
-    const T* uc = static_cast<const T*>(a.uc);
     const T* xt = static_cast<const T*>(a.xt);
     const int i = __ldg(a.nodes + q);
     const int k0 = __ldg(a.rp + i), k1 = __ldg(a.rp + i + 1);
@@ -129,10 +129,9 @@ __device__ __forceinline__ void bgs_node(const BgsArgs& a, long q, int lane) {
 #pragma unroll
         for (int c = 0; c < FB; ++c) drow[c] = __ldg(D + c);
     }
-    // the lane's first block: its column, matrix row, colour test and
-    // aggregate are fixed for the whole cycle, so they are loaded before the
-    // wait on the previous kernel (with programmatic dependent launch they
-    // overlap its tail)
+    // the lane's first block: its column, matrix row and colour test are fixed
+    // for the whole cycle, so they are loaded before the wait on the previous
+    // kernel (with programmatic dependent launch they overlap its tail)
     // (rows hold at least their diagonal block: the clamped index stays in
     // the row, and lanes without a first block load but never use it)
     const int kf = k0 + kk;
@@ -147,14 +146,13 @@ __device__ __forceinline__ void bgs_node(const BgsArgs& a, long q, int lane) {
     // matrix rows are not loaded
     T arf[B];
     if (x_in || lowf) load_row<T, B>(vb + (size_t)(kq - k0) * VS, arf);
-    const int agf = (x_in && uc) ? __ldg(a.agg + jf) : 0;
     if constexpr (PDL) {  // everything below may depend on earlier kernels
         pdl_wait();
         pdl_trigger();
     }
-    const T bi = lane < FB ? ld1<T, CG>(static_cast<const T*>(a.rhs) + (size_t)i * B + f0 + lane) : T(0);
+    const T bi = lane < FB ? ld_cg(static_cast<const T*>(a.rhs) + (size_t)i * B + f0 + lane) : T(0);
     T acc = T(0);
-    if (have) bgs_walk<T, B, FB, CG, G>(a, xt, x_in, uc, vb, VS, k0, kf, k1, jf, lowf, agf, arf, acc);
+    if (have) bgs_walk<T, B, FB, G>(a, xt, x_in, vb, VS, k0, kf, k1, jf, lowf, arf, acc);
     acc = reduce_rows<T, FB>(acc, lane);
     // lanes 0..FB-1: the row sums of A_{f,*} x + A_ff x~ for this node
     T t = T(0);
@@ -165,25 +163,16 @@ __device__ __forceinline__ void bgs_node(const BgsArgs& a, long q, int lane) {
         const T tc = __shfl_sync(0xffffffffu, t, c);
         if (lane < FB) xn = fma(drow[c], tc, xn);
     }
-    if (lane < FB) static_cast<T*>(a.xt)[(size_t)i * FB + lane] = xn;
-    // x_out for node i: every component copied (with the prolongation when
-    // fused), field f corrected by omega x~
+    if (!x_in && lane < FB) static_cast<T*>(a.xt)[(size_t)i * FB + lane] = xn;
+    // x_out for node i: every component copied, field f corrected by omega x~
     const T xf = __shfl_sync(0xffffffffu, xn, (lane - f0) & (kWarp - 1));
-    if (lane < B) {
-        const size_t e = (size_t)i * B + lane;
-        T v = x_in ? ld1<T, CG>(x_in + e) : T(0);
-        if (x_in && uc) v += ld1<T, CG>(uc + (size_t)__ldg(a.agg + i) * B + lane);
-        if (lane >= f0 && lane < f0 + FB) {
-            const T om = a.omega_node ? static_cast<const T*>(a.omega_node)[(size_t)i * a.F + a.field] : T(a.omega);
-            v = fma(om, xf, v);
-        }
-        static_cast<T*>(a.x_out)[e] = v;
-    }
+    if (lane < B)
+        bgs_store<T>(a, x_in, (size_t)i * B + lane, lane >= f0 && lane < f0 + FB, xf, bgs_omega<T>(a, i));
 }
 
 // coarsest level: y_row = sum_c Ainv[row][c] x_c, summed in the inverse's
 // type S; whole warp
-template <typename T, typename S, bool CG>
+template <typename T, typename S>
 __device__ __forceinline__ void gemv_row(int row, int lane, int nd, const S* __restrict__ ainv, const T* x,
                                          T* y) {
     const S* a = ainv + (size_t)row * nd;
@@ -196,12 +185,12 @@ __device__ __forceinline__ void gemv_row(int row, int lane, int nd, const S* __r
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             av[u] = __ldg(a + c + u * kWarp);
-            xv[u] = (S)ld1<T, CG>(x + c + u * kWarp);
+            xv[u] = (S)ld_cg(x + c + u * kWarp);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) acc[u] = fma(av[u], xv[u], acc[u]);
     }
-    for (int u = 0; c < nd; c += kWarp, ++u) acc[u] = fma(__ldg(a + c), (S)ld1<T, CG>(x + c), acc[u]);
+    for (int u = 0; c < nd; c += kWarp, ++u) acc[u] = fma(__ldg(a + c), (S)ld_cg(x + c), acc[u]);
     S sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     sum = warp_sum(sum);
     if (lane == 0) y[row] = (T)sum;
@@ -209,7 +198,7 @@ __device__ __forceinline__ void gemv_row(int row, int lane, int nd, const S* __r
 
 // restriction with R = P^T, P piecewise constant: rc[I,d] = sum_{m in I} res[m,d],
 // members ascending, so the sum order is fixed (deterministic)
-template <typename T, bool CG>
+template <typename T>
 __device__ __forceinline__ void restrict_dof(long t, int b, const int* __restrict__ agg_ptr,
                                              const int* __restrict__ members, const T* res, T* rc) {
     const int I = (int)(t / b);
@@ -220,14 +209,14 @@ __device__ __forceinline__ void restrict_dof(long t, int b, const int* __restric
     for (; q + 4 <= q1; q += 4) {  // four independent loads in flight, added in member order
         const int m0 = __ldg(members + q), m1 = __ldg(members + q + 1);
         const int m2 = __ldg(members + q + 2), m3 = __ldg(members + q + 3);
-        const T v0 = ld1<T, CG>(res + (size_t)m0 * b + d), v1 = ld1<T, CG>(res + (size_t)m1 * b + d);
-        const T v2 = ld1<T, CG>(res + (size_t)m2 * b + d), v3 = ld1<T, CG>(res + (size_t)m3 * b + d);
+        const T v0 = ld_cg(res + (size_t)m0 * b + d), v1 = ld_cg(res + (size_t)m1 * b + d);
+        const T v2 = ld_cg(res + (size_t)m2 * b + d), v3 = ld_cg(res + (size_t)m3 * b + d);
         acc += v0;
         acc += v1;
         acc += v2;
         acc += v3;
     }
-    for (; q < q1; ++q) acc += ld1<T, CG>(res + (size_t)__ldg(members + q) * b + d);
+    for (; q < q1; ++q) acc += ld_cg(res + (size_t)__ldg(members + q) * b + d);
     rc[(size_t)I * b + d] = acc;
 }
 
@@ -237,11 +226,10 @@ __device__ __forceinline__ void restrict_dof(long t, int b, const int* __restric
 template <typename T, int B, int FB, bool FM>
 __global__ void __launch_bounds__(256, 4) spmv_kernel(int n, const int* __restrict__ rp,
                                                    const int* __restrict__ ci,
-                                                   const T* __restrict__ vals, const T* __restrict__ x,
-                                                   const T* __restrict__ rhs, T* __restrict__ y) {
+                                                   const T* __restrict__ vals, const T* x, const T* rhs, T* y) {
     const long i = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (i >= n) return;  // uniform per warp
-    spmv_row<T, B, FB, false, true, FM>(i, threadIdx.x & (kWarp - 1), rp, ci, vals, x, rhs, y);
+    spmv_row<T, B, FB, true, FM>(i, threadIdx.x & (kWarp - 1), rp, ci, vals, x, rhs, y);
 }
 
 template <typename T>
@@ -277,7 +265,7 @@ __global__ void restrict_kernel(int b, int nc, const int* __restrict__ agg_ptr, 
     pdl_wait();
     pdl_trigger();
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < (long)nc * b) restrict_dof<T, false>(t, b, agg_ptr, members, res, rc);
+    if (t < (long)nc * b) restrict_dof<T>(t, b, agg_ptr, members, res, rc);
 }
 
 template <typename T>
@@ -345,7 +333,7 @@ template <typename T, int B, int FB, bool FM>
 __global__ void __launch_bounds__(256, 4) bgs_colour_kernel(BgsArgs a) {
     const long q = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (q >= a.n_in_colour) return;  // uniform per warp
-    bgs_node<T, B, FB, false, true, FM>(a, q, threadIdx.x & (kWarp - 1));
+    bgs_node<T, B, FB, true, FM>(a, q, threadIdx.x & (kWarp - 1));
 }
 
 template <typename T>
@@ -388,7 +376,6 @@ __global__ void __launch_bounds__(W * 32) bgs_wide_kernel(BgsArgs a) {
     const int f0 = a.field * FB;
     const T* __restrict__ vals = static_cast<const T*>(a.vals);
     const T* x_in = static_cast<const T*>(a.x_in);
-    const T* uc = static_cast<const T*>(a.uc);
     const T* xt = static_cast<const T*>(a.xt);
     const int i = __ldg(a.nodes + q);
     const int k0 = __ldg(a.rp + i), k1 = __ldg(a.rp + i + 1);
@@ -408,12 +395,11 @@ __global__ void __launch_bounds__(W * 32) bgs_wide_kernel(BgsArgs a) {
     constexpr int VS = vstride<T, B, FB, FM>();
     T arf[B];
     if (x_in || lowf) load_row<T, B>(vb + (size_t)(kq - k0) * VS, arf);
-    const int agf = (x_in && uc) ? __ldg(a.agg + jf) : 0;
     pdl_wait();
     pdl_trigger();
-    const T bi = (w == 0 && lane < FB) ? static_cast<const T*>(a.rhs)[(size_t)i * B + f0 + lane] : T(0);
+    const T bi = (w == 0 && lane < FB) ? ld_cg(static_cast<const T*>(a.rhs) + (size_t)i * B + f0 + lane) : T(0);
     T acc = T(0);
-    if (have) bgs_walk<T, B, FB, false, W * G>(a, xt, x_in, uc, vb, VS, k0, kf, k1, jf, lowf, agf, arf, acc);
+    if (have) bgs_walk<T, B, FB, W * G>(a, xt, x_in, vb, VS, k0, kf, k1, jf, lowf, arf, acc);
     acc = reduce_rows<T, FB>(acc, lane);
     if (lane < FB) part[w][lane] = acc;
     __syncthreads();
@@ -430,18 +416,10 @@ __global__ void __launch_bounds__(W * 32) bgs_wide_kernel(BgsArgs a) {
         const T tc = __shfl_sync(0xffffffffu, t, c);
         if (lane < FB) xn = fma(drow[c], tc, xn);
     }
-    if (lane < FB) static_cast<T*>(a.xt)[(size_t)i * FB + lane] = xn;
+    if (!x_in && lane < FB) static_cast<T*>(a.xt)[(size_t)i * FB + lane] = xn;
     const T xf = __shfl_sync(0xffffffffu, xn, (lane - f0) & (kWarp - 1));
-    if (lane < B) {
-        const size_t e = (size_t)i * B + lane;
-        T v = x_in ? x_in[e] : T(0);
-        if (x_in && uc) v += uc[(size_t)__ldg(a.agg + i) * B + lane];
-        if (lane >= f0 && lane < f0 + FB) {
-            const T om = a.omega_node ? static_cast<const T*>(a.omega_node)[(size_t)i * a.F + a.field] : T(a.omega);
-            v = fma(om, xf, v);
-        }
-        static_cast<T*>(a.x_out)[e] = v;
-    }
+    if (lane < B)
+        bgs_store<T>(a, x_in, (size_t)i * B + lane, lane >= f0 && lane < f0 + FB, xf, bgs_omega<T>(a, i));
 }
 
 constexpr int kWideWarps = 4;
@@ -493,7 +471,7 @@ __global__ void dense_gemv_kernel(int nd, const S* __restrict__ ainv, const T* _
     pdl_trigger();
     const int row = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (row >= nd) return;
-    gemv_row<T, S, false>(row, threadIdx.x & 31, nd, ainv, x, y);
+    gemv_row<T, S>(row, threadIdx.x & 31, nd, ainv, x, y);
 }
 
 template <typename T, typename S>
@@ -537,23 +515,13 @@ __global__ void __launch_bounds__(256) spmv_tpr_kernel(int n, const int* __restr
     if (act) {
         const int k0 = __ldg(rp + i), k1 = __ldg(rp + i + 1);
         const int kf = k0 + sl;
-        // the first block before the wait (fixed for the cycle)
-        int jf = 0;
-        T af[B];
-        if (kf < k1) {
-            jf = __ldg(ci + kf);
-            load_row<T, B>(vrow<T, B, FB, FM>(vals, k0, k1, kf, r), af);
-        }
+        // (the wait comes before every load but the row range: the gathers go
+        // through L1, whose reuse between the rows of neighbouring nodes is
+        // worth more here than a first block loaded ahead; see pdl_wait)
         pdl_wait();
         pdl_trigger();
-        if (kf < k1) {
-            T xv[B];
-            load_row<T, B>(x + (size_t)jf * B, xv);
-#pragma unroll
-            for (int c = 0; c < B; ++c) acc = fma(af[c], xv[c], acc);
-        }
 #pragma unroll 4
-        for (int k = kf + G; k < k1; k += G) {
+        for (int k = kf; k < k1; k += G) {
             const int j = __ldg(ci + k);
             T a[B], xv[B];
             load_row<T, B>(vrow<T, B, FB, FM>(vals, k0, k1, k, r), a);
@@ -616,28 +584,47 @@ template <typename T, int B, bool FM>
 __global__ void __launch_bounds__(256) residual_upper_kernel(int n, const int* __restrict__ rp,
                                                              const int* __restrict__ ci,
                                                              const unsigned char* __restrict__ lowk,
-                                                             const T* __restrict__ vals, const T* __restrict__ xt,
-                                                             const T* __restrict__ rhs, T omega, T* __restrict__ y) {
+                                                             const T* __restrict__ vals, const T* xt, const T* rhs,
+                                                             T omega, T* y) {
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const int i = (int)(t / B);
     if (i >= n) return;
     const int r = (int)(t - (long)i * B);
     const int k0 = __ldg(rp + i), k1 = __ldg(rp + i + 1);
-    pdl_wait();
-    pdl_trigger();
     T acc = T(0);
-#pragma unroll 4
-    for (int k = k0; k < k1; ++k) {
-        const int j = __ldg(ci + k);
-        if (j == i || __ldg(lowk + k)) continue;
-        T a[B], xv[B];
-        load_row<T, B>(vrow<T, B, B, FM>(vals, k0, k1, k, r), a);
-        load_row<T, B>(xt + (size_t)j * B, xv);
+    bool first = true;
+    // batches of blocks: columns and flags, then rows, then gathers, each
+    // group of loads issued together; the first batch's matrix before the wait
+    constexpr int U = RowBatch<T, B>::kU;
+    for (int k = k0; first || k < k1; k += U) {
+        int j[U];
+        bool on[U];
+        T a[U][B], xv[U][B];
 #pragma unroll
-        for (int c = 0; c < B; ++c) acc = fma(a[c], xv[c], acc);
+        for (int u = 0; u < U; ++u) {
+            j[u] = k + u < k1 ? __ldg(ci + k + u) : i;
+            on[u] = j[u] != i && __ldg(lowk + k + u) == 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (on[u]) load_row<T, B>(vrow<T, B, B, FM>(vals, k0, k1, k + u, r), a[u]);
+        if (first) {
+            first = false;
+            pdl_wait();
+            pdl_trigger();
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (on[u]) load_cg<T, B>(xt + (size_t)j[u] * B, xv[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (on[u]) {
+#pragma unroll
+                for (int c = 0; c < B; ++c) acc = fma(a[u][c], xv[u][c], acc);
+            }
     }
     const size_t e = (size_t)i * B + r;
-    y[e] = (T(1) - omega) * rhs[e] - omega * acc;
+    y[e] = (T(1) - omega) * ld_cg(rhs + e) - omega * acc;
 }
 
 // (one field: the values are block-major, fm is unused)
@@ -678,8 +665,8 @@ struct TprBlock {
 // of the row sum), G * FB threads per node: the G consecutive lanes of scalar
 // row r take every G-th block of the row (G = 1: the whole row), their
 // partial sums meet by a shuffle, and the FB row sums in shared memory for
-// the inverse.  G > 1 shortens each thread's chain of index-then-gather loads
-// (one block row after another), the latency that bounds large colours.
+// the inverse.  Large colours are bound by the bytes in flight: each thread
+// loads its blocks in batches (bgs_row_sum).
 template <typename T, int B, int FB, int G, bool FM>
 __global__ void __launch_bounds__(TprBlock<FB>::kThreads) bgs_tpr_kernel(BgsArgs a) {
     __shared__ T sh_t[TprBlock<FB>::kThreads];
@@ -690,69 +677,33 @@ __global__ void __launch_bounds__(TprBlock<FB>::kThreads) bgs_tpr_kernel(BgsArgs
     const long q = (long)blockIdx.x * (blockDim.x / (FB * G)) + nloc;
     const bool act = q < a.n_in_colour;
     const int f0 = a.field * FB;
-    const T* __restrict__ vals = static_cast<const T*>(a.vals);
-    const T* __restrict__ x_in = static_cast<const T*>(a.x_in);
-    const T* __restrict__ uc = static_cast<const T*>(a.uc);
-    const T* __restrict__ xt = static_cast<const T*>(a.xt);
+    const T* x_in = static_cast<const T*>(a.x_in);
+    const T* xt = static_cast<const T*>(a.xt);
     int i = 0;
-    T t = T(0);
     T acc = T(0);
     if (act) {
         i = __ldg(a.nodes + q);
         const int k0 = __ldg(a.rp + i), k1 = __ldg(a.rp + i + 1);
-        // the first block's static loads before the wait (as in bgs_node)
-        const int kf = k0 + sl;
-        const bool have = kf < k1;
-        const int kq = min(kf, k1 - 1);  // rows hold their diagonal block
-        const int jf = __ldg(a.ci + kq);
-        const bool lowf = __ldg(a.lowk + kq) != 0;
-        const T* vb = vrow<T, B, FB, FM>(vals, k0, k1, k0, f0 + r);
+        const T* vb = vrow<T, B, FB, FM>(static_cast<const T*>(a.vals), k0, k1, k0, f0 + r);
         constexpr int VS = vstride<T, B, FB, FM>();
-        T arf[B];
-        if (x_in || lowf) load_row<T, B>(vb + (size_t)(kq - k0) * VS, arf);
-        const int agf = (x_in && uc) ? __ldg(a.agg + jf) : 0;
-        pdl_wait();
-        pdl_trigger();
-        if (have) {
-            // (a plain loop: the software-pipelined walk of bgs_node needs
-            // more registers, and at this mapping's occupancy that measured
-            // slower on levels far larger than L2)
-            bgs_block<T, B, FB, false>(a, xt, x_in, uc, jf, arf, lowf, agf, acc);
-#pragma unroll(G > 1 ? 8 : 4)
-            for (int k = kf + G; k < k1; k += G) {
-                const bool lower = __ldg(a.lowk + k) != 0;
-                if (!x_in && !lower) continue;
-                const int j = __ldg(a.ci + k);
-                T arow[B];
-                load_row<T, B>(vb + (size_t)(k - k0) * VS, arow);
-                bgs_block<T, B, FB, false>(a, xt, x_in, uc, j, arow, lower, (x_in && uc) ? __ldg(a.agg + j) : 0,
-                                           acc);
-            }
-        }
+        if (x_in) acc = bgs_row_sum<T, B, FB, G, VS, true>(a, xt, x_in, vb, k0, k0 + sl, k1);
+        else acc = bgs_row_sum<T, B, FB, G, VS, false>(a, xt, x_in, vb, k0, k0 + sl, k1);
     }
     if constexpr (G > 1) {  // the G slices of a row are consecutive lanes of one warp
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     }
-    if (act && sl == 0) t = static_cast<const T*>(a.rhs)[(size_t)i * B + f0 + r] - acc;
-    if (sl == 0) sh_t[nloc * FB + r] = t;
+    if (sl == 0) sh_t[nloc * FB + r] = act ? ld_cg(static_cast<const T*>(a.rhs) + (size_t)i * B + f0 + r) - acc : T(0);
     __syncthreads();
     if (!act || sl != 0) return;
     const T* D = static_cast<const T*>(a.dinv) + ((size_t)i * a.F + a.field) * FB * FB + (size_t)r * FB;
     T xn = T(0);
 #pragma unroll
     for (int c = 0; c < FB; ++c) xn = fma(__ldg(D + c), sh_t[nloc * FB + c], xn);
-    static_cast<T*>(a.xt)[(size_t)i * FB + r] = xn;
-    T* __restrict__ x_out = static_cast<T*>(a.x_out);
-    const T om = a.omega_node ? static_cast<const T*>(a.omega_node)[(size_t)i * a.F + a.field] : T(a.omega);
-    const int ag = (x_in && uc) ? __ldg(a.agg + i) : 0;
-    for (int m = 0; m < a.F; ++m) {
-        const size_t e = (size_t)i * B + m * FB + r;
-        T v = x_in ? x_in[e] : T(0);
-        if (x_in && uc) v += uc[(size_t)ag * B + m * FB + r];
-        if (m == a.field) v = fma(om, xn, v);
-        x_out[e] = v;
-    }
+    if (!x_in) static_cast<T*>(a.xt)[(size_t)i * FB + r] = xn;
+    const T om = bgs_omega<T>(a, i);
+    for (int m = 0; m < a.F; ++m)
+        bgs_store<T>(a, x_in, (size_t)i * B + m * FB + r, m == a.field, xn, om);
 }
 
 template <typename T>
@@ -789,17 +740,14 @@ template int launch_bgs_colour_tpr<float>(int, int, const BgsArgs&, cudaStream_t
 // independent vector loads, so each lane has several loads in flight (the
 // four-lanes-per-row mapping has one row load per lane at a time, which
 // bounds large colours by latency).  The FB row sums of the G lanes meet by
-// shuffles within the lane group; lane r < FB finishes row r.  Blocks of
-// higher colour contribute x_in only; x~ is loaded for every block when x_in
-// is set (no branch on the colour flag before the gathers) and used where the
-// flag is set.  XIN: x_in is set.  FB x B <= 16 (the block in registers).
+// shuffles within the lane group; lane r < FB finishes row r.  XIN: x_in is
+// set.  FB x B <= 16 (the block in registers).
 template <typename T, int B, int FB, int G, bool FM, bool XIN>
 __device__ __forceinline__ void bsp_body(const BgsArgs& a, bool act, long q, int s) {
     static_assert(32 % G == 0, "lane groups inside a warp");
     const int f0 = a.field * FB;
     const T* __restrict__ vals = static_cast<const T*>(a.vals);
-    const T* __restrict__ x_in = static_cast<const T*>(a.x_in);
-    const T* __restrict__ uc = static_cast<const T*>(a.uc);
+    const T* x_in = static_cast<const T*>(a.x_in);
     const T* xt = static_cast<const T*>(a.xt);
     T acc[FB];
 #pragma unroll
@@ -816,38 +764,31 @@ __device__ __forceinline__ void bsp_body(const BgsArgs& a, bool act, long q, int
 #pragma unroll 2
         for (int k = k0 + s; k < k1; k += G) {
             const int j = __ldg(a.ci + k);
-            const bool low = __ldg(a.lowk + k) != 0;  // j precedes i in the colour order
-            if (!XIN && !low) continue;
+            if (!XIN && __ldg(a.lowk + k) == 0) continue;  // j does not precede i in the colour order
             T ar[FB][B];
 #pragma unroll
             for (int r = 0; r < FB; ++r) load_row<T, B>(vb + (size_t)(k - k0) * VS + r * B, ar[r]);
-            T tv[FB];
-            load_row<T, FB>(xt + (size_t)j * FB, tv);
             if constexpr (XIN) {
                 T xv[B];
-                load_row<T, B>(x_in + (size_t)j * B, xv);
-                if (uc) {
-                    T pv[B];
-                    load_row<T, B>(uc + (size_t)__ldg(a.agg + j) * B, pv);
-#pragma unroll
-                    for (int c = 0; c < B; ++c) xv[c] += pv[c];
-                }
+                load_cg<T, B>(x_in + (size_t)j * B, xv);
 #pragma unroll
                 for (int r = 0; r < FB; ++r)
 #pragma unroll
                     for (int c = 0; c < B; ++c) acc[r] = fma(ar[r][c], xv[c], acc[r]);
+            } else {
+                T tv[FB];
+                load_cg<T, FB>(xt + (size_t)j * FB, tv);
+#pragma unroll
+                for (int r = 0; r < FB; ++r)
+#pragma unroll
+                    for (int c = 0; c < FB; ++c) {
+                        // column f0 + c of the row, by selects over register indices
+                        T av = ar[r][c];
+#pragma unroll
+                        for (int ff = 1; ff < B / FB; ++ff) av = (ff == a.field) ? ar[r][ff * FB + c] : av;
+                        acc[r] = fma(av, tv[c], acc[r]);
+                    }
             }
-#pragma unroll
-            for (int r = 0; r < FB; ++r)
-#pragma unroll
-                for (int c = 0; c < FB; ++c) {
-                    // column f0 + c of the row, by selects over register indices
-                    T av = ar[r][c];
-#pragma unroll
-                    for (int ff = 1; ff < B / FB; ++ff) av = (ff == a.field) ? ar[r][ff * FB + c] : av;
-                    const T nv = fma(av, tv[c], acc[r]);
-                    acc[r] = low ? nv : acc[r];
-                }
         }
     }
 #pragma unroll
@@ -859,18 +800,11 @@ __device__ __forceinline__ void bsp_body(const BgsArgs& a, bool act, long q, int
     const T* D = static_cast<const T*>(a.dinv) + ((size_t)i * a.F + a.field) * FB * FB + (size_t)s * FB;
     T xn = T(0);
 #pragma unroll
-    for (int c = 0; c < FB; ++c) xn = fma(__ldg(D + c), rhs[c] - acc[c], xn);
-    static_cast<T*>(a.xt)[(size_t)i * FB + s] = xn;
-    T* __restrict__ x_out = static_cast<T*>(a.x_out);
-    const T om = a.omega_node ? static_cast<const T*>(a.omega_node)[(size_t)i * a.F + a.field] : T(a.omega);
-    const int ag = (XIN && uc) ? __ldg(a.agg + i) : 0;
-    for (int m = 0; m < a.F; ++m) {
-        const size_t e = (size_t)i * B + m * FB + s;
-        T v = XIN ? x_in[e] : T(0);
-        if (XIN && uc) v += uc[(size_t)ag * B + m * FB + s];
-        if (m == a.field) v = fma(om, xn, v);
-        x_out[e] = v;
-    }
+    for (int c = 0; c < FB; ++c) xn = fma(__ldg(D + c), ld_cg(rhs + c) - acc[c], xn);
+    if (!XIN) static_cast<T*>(a.xt)[(size_t)i * FB + s] = xn;
+    const T om = bgs_omega<T>(a, i);
+    for (int m = 0; m < a.F; ++m)
+        bgs_store<T>(a, XIN ? x_in : nullptr, (size_t)i * B + m * FB + s, m == a.field, xn, om);
 }
 
 template <typename T, int B, int FB, int G, bool FM>
@@ -1031,42 +965,42 @@ __device__ __forceinline__ void run_phase(const TailPhase& ph, int lane, long gw
         case kPhaseBgs:
             if (HasFm<T, B, FB>::value && ph.bgs.fm)
                 for (long q = gw; q < ph.n; q += W)
-                    bgs_node<T, B, FB, true, false, HasFm<T, B, FB>::value>(ph.bgs, q, lane);
+                    bgs_node<T, B, FB, false, HasFm<T, B, FB>::value>(ph.bgs, q, lane);
             else
-                for (long q = gw; q < ph.n; q += W) bgs_node<T, B, FB, true>(ph.bgs, q, lane);
+                for (long q = gw; q < ph.n; q += W) bgs_node<T, B, FB>(ph.bgs, q, lane);
             break;
         case kPhaseResidual:
             if (HasFm<T, B, FB>::value && ph.fm)
                 for (long i = gw; i < ph.n; i += W)
-                    spmv_row<T, B, FB, true, false, HasFm<T, B, FB>::value>(
+                    spmv_row<T, B, FB, false, HasFm<T, B, FB>::value>(
                         i, lane, ph.rp, ph.ci, static_cast<const T*>(ph.vals), static_cast<const T*>(ph.x),
                         static_cast<const T*>(ph.rhs), static_cast<T*>(ph.y));
             else
                 for (long i = gw; i < ph.n; i += W)
-                    spmv_row<T, B, FB, true>(i, lane, ph.rp, ph.ci, static_cast<const T*>(ph.vals),
+                    spmv_row<T, B, FB>(i, lane, ph.rp, ph.ci, static_cast<const T*>(ph.vals),
                                              static_cast<const T*>(ph.x), static_cast<const T*>(ph.rhs),
                                              static_cast<T*>(ph.y));
             break;
         case kPhaseRestrict:
             for (long t = gt; t < (long)ph.n * B; t += NT)
-                restrict_dof<T, true>(t, B, ph.rp, ph.ci, static_cast<const T*>(ph.x), static_cast<T*>(ph.y));
+                restrict_dof<T>(t, B, ph.rp, ph.ci, static_cast<const T*>(ph.x), static_cast<T*>(ph.y));
             break;
         case kPhaseGemv:
             for (long row = gw; row < ph.n; row += W)
-                gemv_row<T, double, true>((int)row, lane, ph.n, static_cast<const double*>(ph.vals),
+                gemv_row<T, double>((int)row, lane, ph.n, static_cast<const double*>(ph.vals),
                                           static_cast<const T*>(ph.x), static_cast<T*>(ph.y));
             break;
         case kPhaseGemv32:
             for (long row = gw; row < ph.n; row += W)
-                gemv_row<T, float, true>((int)row, lane, ph.n, static_cast<const float*>(ph.vals),
+                gemv_row<T, float>((int)row, lane, ph.n, static_cast<const float*>(ph.vals),
                                          static_cast<const T*>(ph.x), static_cast<T*>(ph.y));
             break;
         case kPhaseProlongCopy:  // y = x + P uc over n fine nodes (x may equal y); uc in rhs, agg in ci
             for (long e = gt; e < (long)ph.n * B; e += NT) {
                 const int i = (int)(e / B), d = (int)(e - (long)i * B);
                 static_cast<T*>(ph.y)[e] =
-                    ld1<T, true>(static_cast<const T*>(ph.x) + e) +
-                    ld1<T, true>(static_cast<const T*>(ph.rhs) + (size_t)__ldg(ph.ci + i) * B + d);
+                    ld_cg(static_cast<const T*>(ph.x) + e) +
+                    ld_cg(static_cast<const T*>(ph.rhs) + (size_t)__ldg(ph.ci + i) * B + d);
             }
             break;
         case kPhaseZero:

@@ -123,9 +123,8 @@ __global__ void __launch_bounds__(StagedShape<FB>::kThreads) bgs_staged_kernel(B
     const int w = tid - nloc * (FB * G);
     const int r = w / G, sl = w - r * G;
     const int f0 = a.field * FB;
-    const T* __restrict__ x_in = static_cast<const T*>(a.x_in);
-    const T* __restrict__ uc = static_cast<const T*>(a.uc);
-    const T* __restrict__ xt = static_cast<const T*>(a.xt);
+    const T* x_in = static_cast<const T*>(a.x_in);
+    const T* xt = static_cast<const T*>(a.xt);
     const long first = (long)blockIdx.x * batches_per_cta * NB;
     long nbatch = ((long)a.n_in_colour - first + NB - 1) / NB;
     if (nbatch > batches_per_cta) nbatch = batches_per_cta;
@@ -176,31 +175,22 @@ __global__ void __launch_bounds__(StagedShape<FB>::kThreads) bgs_staged_kernel(B
                 const int j = crow[kk];
                 T arow[B];
                 load_row<T, B>(vrow0 + (size_t)kk * VS + roff, arow);
-                bgs_block<T, B, FB, false>(a, xt, x_in, uc, j, arow, lower, (x_in && uc) ? __ldg(a.agg + j) : 0,
-                                           acc);
+                bgs_block<T, B, FB>(a, xt, x_in, j, arow, lower, acc);
             }
         }
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (sl == 0) sh_t[nloc * FB + r] = act ? static_cast<const T*>(a.rhs)[(size_t)i * B + f0 + r] - acc : T(0);
+        if (sl == 0) sh_t[nloc * FB + r] = act ? ld_cg(static_cast<const T*>(a.rhs) + (size_t)i * B + f0 + r) - acc : T(0);
         __syncthreads();  // the row sums are in sh_t; every thread is done with stage st
         if (act && sl == 0) {
             const T* D = static_cast<const T*>(a.dinv) + ((size_t)i * a.F + a.field) * FB * FB + (size_t)r * FB;
             T xn = T(0);
 #pragma unroll
             for (int c = 0; c < FB; ++c) xn = fma(__ldg(D + c), sh_t[nloc * FB + c], xn);
-            static_cast<T*>(a.xt)[(size_t)i * FB + r] = xn;
-            T* __restrict__ x_out = static_cast<T*>(a.x_out);
-            const T om =
-                a.omega_node ? static_cast<const T*>(a.omega_node)[(size_t)i * a.F + a.field] : T(a.omega);
-            const int ag = (x_in && uc) ? __ldg(a.agg + i) : 0;
-            for (int m = 0; m < a.F; ++m) {
-                const size_t e = (size_t)i * B + m * FB + r;
-                T v = x_in ? x_in[e] : T(0);
-                if (x_in && uc) v += uc[(size_t)ag * B + m * FB + r];
-                if (m == a.field) v = fma(om, xn, v);
-                x_out[e] = v;
-            }
+            if (!x_in) static_cast<T*>(a.xt)[(size_t)i * FB + r] = xn;
+            const T om = bgs_omega<T>(a, i);
+            for (int m = 0; m < a.F; ++m)
+                bgs_store<T>(a, x_in, (size_t)i * B + m * FB + r, m == a.field, xn, om);
         }
         issue(t + kStagedStages);  // refill stage st (its reads ended at the barrier above)
         __syncthreads();        // sh_t is reused by the next batch

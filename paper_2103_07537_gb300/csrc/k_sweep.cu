@@ -82,9 +82,11 @@ __global__ void __launch_bounds__(SweepShape<FB>::kThreads) bgs_sweep_kernel(Bgs
     const int nc = sw.c_hi - sw.c_lo;
     const int f0 = a.field * FB;
     const T* __restrict__ vals = static_cast<const T*>(a.vals);
-    const T* __restrict__ x_in = static_cast<const T*>(a.x_in);
-    const T* __restrict__ uc = static_cast<const T*>(a.uc);
-    const T* xt = static_cast<const T*>(a.xt);  // written in this launch: read through L2
+    // x_in and x~ are written in this launch: read through L2.  (A node updates
+    // its entries of x_in only once its lower-colour neighbours are done, so
+    // none of them still reads the entries before the update.)
+    const T* x_in = static_cast<const T*>(a.x_in);
+    const T* xt = static_cast<const T*>(a.xt);
     // colour and tile ranges of the step (fixed for the level)
     for (int q = tid; q <= nc; q += NT) {
         s_cptr[q] = __ldg(sw.colour_ptr + sw.c_lo + q);
@@ -151,33 +153,24 @@ __global__ void __launch_bounds__(SweepShape<FB>::kThreads) bgs_sweep_kernel(Bgs
                     const int j = __ldg(a.ci + k);
                     T arow[B];
                     load_row<T, B>(vb + (size_t)(k - k0) * VS, arow);
-                    bgs_block<T, B, FB, true, false>(a, xt, x_in, uc, j, arow, lower,
-                                                     (x_in && uc) ? __ldg(a.agg + j) : 0, acc);
+                    bgs_block<T, B, FB>(a, xt, x_in, j, arow, lower, acc);
                 }
             }
             if constexpr (G > 1) {  // the G slices of a row are consecutive lanes of one warp
 #pragma unroll
                 for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             }
-            if (sl == 0) sh_t[nloc * FB + r] = (act ? static_cast<const T*>(a.rhs)[(size_t)i * B + f0 + r] - acc : T(0));
+            if (sl == 0) sh_t[nloc * FB + r] = (act ? ld_cg(static_cast<const T*>(a.rhs) + (size_t)i * B + f0 + r) - acc : T(0));
             __syncthreads();
             if (act && sl == 0) {
                 const T* D = static_cast<const T*>(a.dinv) + ((size_t)i * a.F + a.field) * FB * FB + (size_t)r * FB;
                 T xn = T(0);
 #pragma unroll
                 for (int c = 0; c < FB; ++c) xn = fma(__ldg(D + c), sh_t[nloc * FB + c], xn);
-                static_cast<T*>(a.xt)[(size_t)i * FB + r] = xn;
-                T* __restrict__ x_out = static_cast<T*>(a.x_out);
-                const T om =
-                    a.omega_node ? static_cast<const T*>(a.omega_node)[(size_t)i * a.F + a.field] : T(a.omega);
-                const int ag = (x_in && uc) ? __ldg(a.agg + i) : 0;
-                for (int m = 0; m < a.F; ++m) {
-                    const size_t e = (size_t)i * B + m * FB + r;
-                    T v = x_in ? x_in[e] : T(0);
-                    if (x_in && uc) v += uc[(size_t)ag * B + m * FB + r];
-                    if (m == a.field) v = fma(om, xn, v);
-                    x_out[e] = v;
-                }
+                if (!x_in) static_cast<T*>(a.xt)[(size_t)i * FB + r] = xn;
+                const T om = bgs_omega<T>(a, i);
+                for (int m = 0; m < a.F; ++m)
+                    bgs_store<T>(a, x_in, (size_t)i * B + m * FB + r, m == a.field, xn, om);
             }
             __syncthreads();  // sh_t is reused by the next pass
         }
