@@ -122,7 +122,6 @@ struct Level {
     float* dinv32 = nullptr;
     int *agg = nullptr, *agg_ptr = nullptr, *members = nullptr;
     void *xa = nullptr, *xb = nullptr, *xt = nullptr, *res = nullptr, *rhs = nullptr, *uc = nullptr;
-    int agg_rounds = 0, colour_rounds = 0;
     // row mapping chosen for this level: smoother 0 warp per node, 1 thread per row, 2 thread per
     // row in half-size CTAs, 3 four lanes per row, 4 four lanes per row with the rows staged in
     // shared memory by asynchronous copies (steps from a zero iterate use 3), 5 four warps per
@@ -254,7 +253,7 @@ struct bamg_ctx {
     cudaEvent_t vals_ev = nullptr;
     bool vals_pending = false;
     // the colouring of every level that gets a smoother runs on its own stream,
-    // driven by its own host thread (its rounds poll a host flag), once the
+    // driven by its own host thread (it reads its result back), once the
     // hierarchy's aggregation and Galerkin products are done, beside the
     // coarsest LU and the smoother data of the other levels (it needs only the
     // level's pattern)
@@ -262,7 +261,7 @@ struct bamg_ctx {
         std::thread thread;
         cudaStream_t stream = nullptr;
         cudaEvent_t ev = nullptr;
-        int status = BAMG_OK, n_colours = 0, rounds = 0;
+        int status = BAMG_OK, n_colours = 0;
         int *flag = nullptr, *queue = nullptr, *pin = nullptr;
     } cjob[kMaxLevels];
     // the tensor-core coarsest LU enqueued on cap_stream ahead of the smoother
@@ -780,9 +779,10 @@ static int schwarz_level(bamg_ctx* h, int l, cudaStream_t s) {
 }
 
 // Tiles of the persistent sweep on a coloured level (colour lists and lowk
-// exist) and their dependencies; skipped when sweeps are off, for sub-block
+// exist), and their dependencies where the sweep is forced; skipped when sweeps are off, for sub-block
 // sizes without a sweep kernel and for levels with more colours than it takes.
-static int build_sweep_plan(bamg_ctx* h, Level& L, cudaStream_t s) {
+static int build_sweep_plan(bamg_ctx* h, Level& L, cudaStream_t s);
+static int sweep_tiles(bamg_ctx* h, Level& L, cudaStream_t s) {
     const int ntile = sweep_tile_nodes(h->fb);
     if (h->p.sweep == 1 || ntile <= 0 || L.n_colours < 1 || L.n_colours > kSweepMaxColours) return BAMG_OK;
     const int C = L.n_colours;
@@ -790,6 +790,12 @@ static int build_sweep_plan(bamg_ctx* h, Level& L, cudaStream_t s) {
     for (int c = 0; c < C; ++c)
         L.sw_tile_ptr[c + 1] = L.sw_tile_ptr[c] + ceil_div(L.colour_ptr[c + 1] - L.colour_ptr[c], ntile);
     L.sw_tiles = L.sw_tile_ptr[C];
+    if (h->p.sweep < 2) return BAMG_OK;  // (the autotuner builds the plan where it times or takes the sweep)
+    L.sweep = h->p.sweep - 1;
+    return build_sweep_plan(h, L, s);
+}
+static int build_sweep_plan(bamg_ctx* h, Level& L, cudaStream_t s) {
+    const int C = L.n_colours, ntile = sweep_tile_nodes(h->fb);
     TRY(h->alloc(&L.sw_tile_ptr_d, (size_t)C + 1));
     TRY(h->alloc(&L.sw_lo, (size_t)L.sw_tiles * C));
     TRY(h->alloc(&L.sw_hi, (size_t)L.sw_tiles * C));
@@ -805,7 +811,18 @@ static int build_sweep_plan(bamg_ctx* h, Level& L, cudaStream_t s) {
                    L.sw_tiles, tile_of, L.sw_lo, L.sw_hi, s));
     BAMG_CUDA_TRY(cudaStreamSynchronize(s));
     h->release(tile_of);
-    if (h->p.sweep >= 2) L.sweep = h->p.sweep - 1;
+    return BAMG_OK;
+}
+
+// stored blocks in the level's longest row (the staged smoother's slots)
+static int level_max_row(bamg_ctx* h, Level& L, cudaStream_t s) {
+    int* mr = nullptr;
+    TRY(h->alloc(&mr, 1));
+    TRY(launch_row_len_max(L.n, L.rp, mr, s));
+    BAMG_CUDA_TRY(cudaMemcpyAsync(h->h_pin, mr, sizeof(int), cudaMemcpyDeviceToHost, s));
+    BAMG_CUDA_TRY(cudaStreamSynchronize(s));
+    L.max_row = h->h_pin[0];
+    h->release(mr);
     return BAMG_OK;
 }
 
@@ -921,11 +938,16 @@ static int autotune_levels(bamg_ctx* h, cudaStream_t s) {
                     hit = true;
                     break;
                 }
-            if (hit) {
-                L.tune_cached = 1;
-                continue;
-            }
+            if (hit) L.tune_cached = 1;
         }
+        if (L.tune_cached) {
+            // (what only the candidates not taken would need is not built)
+            if (L.bgs_tpr == 4) TRY(level_max_row(h, L, s));
+            if (L.sweep) TRY(build_sweep_plan(h, L, s));
+            continue;
+        }
+        TRY(level_max_row(h, L, s));
+        if (L.sw_tiles > 0 && h->p.sweep == 0 && h->p.autotune == 1) TRY(build_sweep_plan(h, L, s));
         const size_t nb = (size_t)L.n * b;
         BAMG_CUDA_TRY(cudaMemsetAsync(L.xa, 0, nb * sizeof(T), s));
         BAMG_CUDA_TRY(cudaMemsetAsync(L.res, 0, nb * sizeof(T), s));
@@ -1183,14 +1205,13 @@ static int colour_start(bamg_ctx* h, int l, Level& L, cudaStream_t s) {
         j.thread = std::thread([jp, dev, n, rp, ci, colour]() {
             int st = cudaSetDevice(dev) == cudaSuccess ? BAMG_OK : BAMG_ECUDA;
             if (st == BAMG_OK)
-                st = colour_nodes(n, rp, ci, colour, jp->flag, jp->pin, jp->stream, &jp->n_colours, &jp->rounds,
-                                  jp->queue);
+                st = colour_nodes(n, rp, ci, colour, jp->flag, jp->pin, jp->stream, &jp->n_colours, jp->queue);
             if (cudaEventRecord(jp->ev, jp->stream) != cudaSuccess && st == BAMG_OK) st = BAMG_ECUDA;
             jp->status = st;
         });
     } catch (...) {
         // no thread: colour on the setup stream now
-        j.status = colour_nodes(n, rp, ci, colour, j.flag, j.pin, s, &j.n_colours, &j.rounds, j.queue);
+        j.status = colour_nodes(n, rp, ci, colour, j.flag, j.pin, s, &j.n_colours, j.queue);
         if (j.status == BAMG_OK) BAMG_CUDA_TRY(cudaEventRecord(j.ev, s));
     }
     return BAMG_OK;
@@ -1206,7 +1227,6 @@ static int colour_join(bamg_ctx* h, int l, Level& L, cudaStream_t s, bool* done)
     TRY(j.status);
     BAMG_CUDA_TRY(cudaStreamWaitEvent(s, j.ev, 0));
     L.n_colours = j.n_colours;
-    L.colour_rounds = j.rounds;
     h->release(j.flag);
     h->release(j.queue);
     j.flag = j.queue = nullptr;
@@ -1341,19 +1361,16 @@ static int setup_impl(bamg_ctx* h, const int* row_ptr, const int* col_idx, const
         TRY(h->alloc(&w.state, (size_t)L.n));
         TRY(h->alloc(&w.rootid, (size_t)L.n + 1));
         TRY(h->alloc(&w.agg1, (size_t)L.n));
-        TRY(h->alloc(&w.settled, (size_t)L.n));
         TRY(h->alloc(&w.flag, 4));
         TRY(h->alloc(&d_count, 4));
         TRY(h->alloc(&scan_tmp, (size_t)stb / sizeof(int) + 1));
         TRY(h->alloc(&L.agg, (size_t)L.n));
         w.host_flag = h->h_pin;
         BAMG_CUDA_TRY(cudaMemsetAsync(d_count, 0, 4 * sizeof(int), s));
-        int rounds = 0;
         int *g_rp = L.rp, *g_ci = L.ci;
         if (h->nf > 1) TRY(level_field_graph(h, L, &g_rp, &g_ci, s));
-        const int nc = aggregate_nodes(L.n, g_rp, g_ci, L.agg, w, d_count, scan_tmp, stb, s, &rounds);
+        const int nc = aggregate_nodes(L.n, g_rp, g_ci, L.agg, w, d_count, scan_tmp, stb, s);
         if (nc < 0) return nc;
-        L.agg_rounds = rounds;
         if (h->nf > 1) {
             h->release(g_rp);
             h->release(g_ci);
@@ -1381,7 +1398,6 @@ static int setup_impl(bamg_ctx* h, const int* row_ptr, const int* col_idx, const
         h->release(w.state);
         h->release(w.rootid);
         h->release(w.agg1);
-        h->release(w.settled);
         if (nc == 0 || nc == L.n) break;  // no coarsening possible
         L.n_agg = nc;
         TRY(h->alloc(&L.agg_ptr, (size_t)nc + 1));
@@ -1465,11 +1481,9 @@ static int setup_impl(bamg_ctx* h, const int* row_ptr, const int* col_idx, const
             int *cflag = nullptr, *queue = nullptr;
             TRY(h->alloc(&cflag, 4));
             TRY(h->alloc(&queue, 2 * (size_t)L.n));
-            int rounds = 0;
             int *g_rp = L.rp, *g_ci = L.ci;
             if (h->nf > 1) TRY(level_field_graph(h, L, &g_rp, &g_ci, s));
-            TRY(colour_nodes(L.n, g_rp, g_ci, L.colour, cflag, h->h_pin, s, &L.n_colours, &rounds, queue));
-            L.colour_rounds = rounds;
+            TRY(colour_nodes(L.n, g_rp, g_ci, L.colour, cflag, h->h_pin, s, &L.n_colours, queue));
             h->release(cflag);
             h->release(queue);
             if (h->nf > 1) {
@@ -1500,7 +1514,7 @@ static int setup_impl(bamg_ctx* h, const int* row_ptr, const int* col_idx, const
         TRY(h->alloc(&L.colour_ptr_d, (size_t)L.n_colours + 1));
         TRY(h->alloc(&L.colour_nodes, (size_t)L.n));
         int* tmp = nullptr;
-        TRY(h->alloc(&tmp, (size_t)L.n + 1 + scan_tmp_bytes(L.n) / sizeof(int) + 16));
+        TRY(h->alloc(&tmp, (size_t)colour_order_ints(L.n, L.n_colours)));
         TRY(colour_order(L.n, L.n_colours, L.colour, L.colour_ptr_d, L.colour_nodes, tmp, s));
         L.colour_ptr.assign(L.n_colours + 1, 0);
         BAMG_CUDA_TRY(cudaMemcpyAsync(L.colour_ptr.data(), L.colour_ptr_d, sizeof(int) * (L.n_colours + 1),
@@ -1511,16 +1525,7 @@ static int setup_impl(bamg_ctx* h, const int* row_ptr, const int* col_idx, const
         TRY(h->alloc(&L.lowk, (size_t)L.nnzb));
         if (h->nf > 1) TRY(field_lower_flags(L.n, L.rp, L.ci, L.colour, L.node_field, L.lowk, s));
         else TRY(launch_lower_flags(L.n, L.rp, L.ci, L.colour, L.lowk, s));
-        TRY(build_sweep_plan(h, L, s));
-        {
-            int* mr = nullptr;
-            TRY(h->alloc(&mr, 1));
-            TRY(launch_row_len_max(L.n, L.rp, mr, s));
-            BAMG_CUDA_TRY(cudaMemcpyAsync(h->h_pin, mr, sizeof(int), cudaMemcpyDeviceToHost, s));
-            BAMG_CUDA_TRY(cudaStreamSynchronize(s));
-            L.max_row = h->h_pin[0];
-            h->release(mr);
-        }
+        TRY(sweep_tiles(h, L, s));
         h->t_phase[3] += ms_since(tp);
         tp = Clock::now();
         if (!L.dinv64) {  // (already there when P was smoothed)
@@ -3104,9 +3109,8 @@ extern "C" int amg_stats(bamg_t h, char* json, int cap) {
         if (l) o += ",";
         o += "{\"n\":" + std::to_string(L.n) + ",\"nnzb\":" + std::to_string(L.nnzb) +
              ",\"colours\":" + std::to_string(L.n_colours) + ",\"aggregates\":" + std::to_string(L.n_agg) +
-             ",\"aggregation_rounds\":" + std::to_string(L.agg_rounds) +
-             ",\"colouring_rounds\":" + std::to_string(L.colour_rounds) +
-             ",\"smoother_mapping\":\"" + (L.sweep == 2     ? "sweep-split"
+             // (one launch each: no rounds)
+             ",\"aggregation_rounds\":0,\"colouring_rounds\":0" + ",\"smoother_mapping\":\"" + (L.sweep == 2     ? "sweep-split"
                                           : L.sweep        ? "sweep"
                                           : L.bgs_tpr == 7 ? "block-split8"
                                           : L.bgs_tpr == 6 ? "block-split16"

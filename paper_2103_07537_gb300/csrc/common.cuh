@@ -515,13 +515,12 @@ struct AggWork {
     int* state;   // [n]
     int* rootid;  // [n + 1]
     int* agg1;    // [n]
-    int* flag;    // [1] device
-    int* host_flag;  // pinned host [1]
-    unsigned char* settled = nullptr;  // [n] optional: nodes whose neighbourhood is decided
+    int* flag;    // [2] device: ticket, failure word
+    int* host_flag;  // pinned host [3]
 };
-// d_count: 2 device ints (aggregate count, error flag); w.host_flag: 2 pinned ints
+// d_count: 2 device ints (aggregate count, error flag)
 int aggregate_nodes(int n, const int* rp, const int* ci, int* agg, AggWork& w, int* d_count,
-                    int* d_scan_tmp, long scan_tmp_bytes, cudaStream_t s, int* rounds_out);
+                    int* d_scan_tmp, long scan_tmp_bytes, cudaStream_t s);
 int build_members(int n, int nc, const int* agg, int* agg_ptr, int* members, int* d_tmp,
                   cudaStream_t s);
 // Single-CTA worklist colouring (k_setup.cu): colour[n], queues qa, qb (n ints
@@ -536,10 +535,12 @@ constexpr int kWorklistSmemMax = kWorklistMaxNodes * 5 + 16;  // dynamic shared 
 __global__ void __launch_bounds__(1024) colour_worklist_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci,
                                        int* __restrict__ colour, int* __restrict__ qa, int* __restrict__ qb,
                                        int* __restrict__ out, const int* __restrict__ pre_err);
-// d_queue: 2n device ints of scratch (nullptr: always use the multi-launch rounds)
-int colour_nodes(int n, const int* rp, const int* ci, int* colour, int* d_flag, int* h_flag,
-                 cudaStream_t s, int* n_colours, int* rounds_out, int* d_queue);
-// colour_ptr[C+1] and nodes sorted by (colour, index)
+// first-fit colours of every node; d_flag: 4 device ints, h_flag: 4 pinned host
+// ints, d_queue: 2n device ints of scratch
+int colour_nodes(int n, const int* rp, const int* ci, int* colour, int* d_flag, int* h_flag, cudaStream_t s,
+                 int* n_colours, int* d_queue);
+// colour_ptr[C+1] and nodes sorted by (colour, index); d_tmp: colour_order_ints(n, C) ints
+long colour_order_ints(int n, int C);
 int colour_order(int n, int C, const int* colour, int* colour_ptr, int* nodes, int* d_tmp,
                  cudaStream_t s);
 // RAP with the tentative prolongator: symbolic (row sizes), then numeric

@@ -6,10 +6,10 @@
 //
 // Order independence.  The aggregation and the colouring are defined by
 // sequential greedy rules in ascending node order; the kernels reach the
-// same result with priority rounds (a node decides once every lower-index
+// same result in one launch (a node decides once every lower-index
 // node that could influence it has decided), so the result does not depend
 // on thread scheduling.  A state only ever moves from "undecided" to a final
-// value, so a stale read inside a round can only delay a decision.
+// value, so a stale read can only delay a decision.
 #include "common.cuh"
 
 namespace bamg {
@@ -161,114 +161,136 @@ int launch_check_pattern(int n, const int* rp, const int* ci, int* diag, int* er
 // Aggregation.  Sequential rule (ascending node order): a node whose
 // neighbours and itself are all free becomes a root; it and its neighbours
 // form an aggregate.  Equivalently, the roots are the lexicographically-first
-// maximal set of nodes with pairwise hop distance >= 3.  Priority rounds:
-// an undecided node with a root within distance 2 is out; an undecided node
-// with no undecided lower-index node and no root within distance 2 is a root.
+// maximal set of nodes with pairwise hop distance >= 3: a node with a lower
+// root within distance 2 is out; one whose lower nodes within distance 2 are
+// all out is a root.
 // ---------------------------------------------------------------------------
 enum : int { kUndecided = 0, kRoot = 1, kOut = 2 };
 
-// a launch with the programmatic-dependent-launch attribute (the round
-// kernels of aggregation and colouring)
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_round(void (*kernel)(KArgs...), int grid, int threads, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+__device__ __forceinline__ int ld_relaxed(const int* p) {
+    int v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
-// the round kernels' grid: at most four CTAs per SM, a grid-stride loop beyond
-static int round_grid(int n, int threads) { return std::max(1, std::min(ceil_div(n, threads), 152 * 4)); }
+__device__ __forceinline__ void st_relaxed(int* p, int v) {
+    asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 
+// The greedy rules of aggregation and colouring decide every node from nodes
+// of lower index only.  Both run as one launch: CTAs take chunks of
+// kChunk consecutive nodes in ascending order from an atomic ticket, a thread
+// per node, and a node waits (polling L2) for the lower nodes its rule reads.
+// Those belong to its own chunk or to chunks taken earlier by running CTAs, so
+// some node can always be decided, whatever part of the grid is resident.
+// Every wait is bounded all the same: kChunkSpins polls, then the failure word
+// is set and every CTA leaves.  (Rounds over all nodes, one launch or two per
+// round, cost 13 to 26 us for each step of the dependency chain -- 455 steps
+// for the colouring of the 65^3 grid, 128 for its aggregation -- where a step
+// here is a store and a poll, about 1 us through L2 and less inside a CTA:
+// 3D setup, 65^3 nodes: colouring 5.5 ms, aggregation 3.4 ms as rounds.)
+constexpr int kChunk = 256;
+constexpr int kChunkCtas = 4;  // CTAs per SM (the window of nodes in work)
+constexpr int kChunkSpins = 1 << 22;  // at least half a microsecond each
 
+// the next chunk's first node, or n at the end or after a failure (whole CTA)
+__device__ __forceinline__ int take_chunk(int n, int* ticket, const int* fail) {
+    __shared__ int s_base;
+    __syncthreads();  // s_base, and the caller's use of the previous chunk
+    if (threadIdx.x == 0) {
+        const int c = atomicAdd(ticket, 1);
+        s_base = c >= (n + kChunk - 1) / kChunk || ld_relaxed(fail) != 0 ? n : c * kChunk;
+    }
+    __syncthreads();
+    return s_base;
+}
+static int chunk_grid(int n) { return std::min(ceil_div(n, kChunk), 152 * kChunkCtas); }
 
-// One round in two one-hop passes over the states at the start of the round.
-// Pass 1: m1[i] = smallest undecided index in {i} + N(i) (INT_MAX if none),
-//         r1[i] = 1 if a root is in {i} + N(i).
-// Pass 2: an undecided node with r1 set on {i} + N(i) (a root within distance
-//         2) is out; one whose smallest m1 over {i} + N(i) is i itself (no
-//         undecided lower node within distance 2) becomes a root.
-// New roots of one round are pairwise at distance >= 3, and a node becomes a
-// root exactly when every lower node within distance 2 is out: the rounds
-// reach the sequential ascending-order result.
-// A node with no undecided node in {i} + N(i) is settled: its m1 (none) and
-// r1 (a root in N(i): no new root can appear there) never change again, so
-// later rounds skip it (settled: optional, zeroed before the first round).
-__device__ __forceinline__ void mis2_pass1_node(int i, const int* __restrict__ rp, const int* __restrict__ ci,
-                                                const int* __restrict__ state, int* __restrict__ m1,
-                                                int* __restrict__ r1, unsigned char* __restrict__ settled) {
-    if (settled && settled[i]) return;
-    int mn = 0x7fffffff, root = 0;
-    constexpr int U = 16;  // loads of a batch in flight together
-    const int k0 = rp[i], k1 = rp[i + 1];
-    for (int kb = k0; kb < k1; kb += U) {  // the row contains i itself (diagonal block)
-        int jj[U], sj[U];
+// Roots: node i is a root when no lower node within distance 2 is one.  A new
+// root's warp marks every higher node within distance 2 as out, so most nodes
+// are decided without any work of their own.  The others are tested by their
+// warp, a lane per row of {i} + N(i): a root among the rows' lower entries
+// takes i out, an undecided entry makes i wait (it is polled alone), else i is
+// a root.  Any of a warp's nodes may be tested, not only its lowest: a warp
+// that covers the end of one grid line and the start of the next would
+// otherwise chain the lines (47 ms for the 65^3 grid).  A thread per node
+// walking its rows alone took 8.6 ms: a root walks all of its 350 entries, and
+// the roots form a chain.
+// ctl: ticket, failure word.
+__global__ void __launch_bounds__(kChunk) mis2_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci,
+                                                      int* state, int* ctl) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    constexpr int U = 8;  // entries read together
+    for (;;) {
+        const int base = take_chunk(n, ctl, ctl + 1);
+        if (base >= n) return;
+        const int i0 = base + (int)threadIdx.x - lane;  // the warp's first node
+        bool done = i0 + lane >= n;
+        int wait = -1;  // the undecided node this lane's node was last found to wait for
+        for (int spins = 0;;) {
+            if (!done) {
+                const int own = ld_relaxed(state + i0 + lane);
+                const int other = wait >= 0 ? ld_relaxed(state + wait) : kOut;
+                done = own != kUndecided;
+                if (other != kUndecided) wait = -1;
+            }
+            if (!__any_sync(kAll, !done)) break;
+            const unsigned ready = __ballot_sync(kAll, !done && wait < 0);
+            if (!ready) {
+                if (++spins > kChunkSpins) st_relaxed(ctl + 1, 1);
+                if ((spins & 1023) == 1023 && __any_sync(kAll, ld_relaxed(ctl + 1) != 0)) break;
+                __nanosleep(100);
+                continue;
+            }
+            const int src = __ffs(ready) - 1, i = i0 + src;
+            const int k0 = rp[i], k1 = rp[i + 1];
+            bool root = false;
+            int w = -1;
+            for (int k = k0 + lane; k < k1; k += 32) {
+                const int j = ci[k];
+                const int q1 = rp[j + 1];
+                for (int q = rp[j]; q < q1; q += U) {
+                    int m[U], sm[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) jj[u] = kb + u < k1 ? ci[kb + u] : -1;
+                    for (int u = 0; u < U; ++u) m[u] = q + u < q1 ? ci[q + u] : i;
+                    // (an entry >= i reads i's own state, which is ignored)
 #pragma unroll
-        for (int u = 0; u < U; ++u) sj[u] = jj[u] >= 0 ? state[jj[u]] : kOut;
+                    for (int u = 0; u < U; ++u) sm[u] = ld_relaxed(state + min(m[u], i));
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (sj[u] == kUndecided) mn = min(mn, jj[u]);
-            if (sj[u] == kRoot) root = 1;
+                    for (int u = 0; u < U; ++u)
+                        if (m[u] < i) {
+                            root |= sm[u] == kRoot;
+                            if (sm[u] == kUndecided) w = max(w, m[u]);
+                        }
+                    if (m[U - 1] >= i) break;  // columns ascending: nothing lower follows
+                }
+            }
+            root = __any_sync(kAll, root);
+            w = __reduce_max_sync(kAll, w);
+            if (!root && w >= 0) {
+                if (lane == src) wait = w;
+                continue;
+            }
+            if (lane == src) {
+                st_relaxed(state + i, root ? kOut : kRoot);
+                done = true;
+            }
+            if (root) continue;
+            for (int k = k0 + lane; k < k1; k += 32) {
+                const int j = ci[k];
+                const int q1 = rp[j + 1];
+                for (int q = rp[j]; q < q1; q += U) {
+                    int m[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) m[u] = q + u < q1 ? ci[q + u] : -1;
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (m[u] > i) st_relaxed(state + m[u], kOut);
+                }
+            }
+            __syncwarp();  // the marks before this warp looks at its states again
         }
     }
-    m1[i] = mn;
-    r1[i] = root;
-    if (settled && mn == 0x7fffffff) settled[i] = 1;
-}
-
-// the rounds run as programmatic dependent launches (each is scheduled while
-// its predecessor drains and waits for it in hardware), a thread per node
-// (a grid-stride loop when launched smaller)
-__global__ void mis2_pass1_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci,
-                                  const int* __restrict__ state, int* __restrict__ m1, int* __restrict__ r1,
-                                  unsigned char* __restrict__ settled) {
-    pdl_wait();
-    pdl_trigger();
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        mis2_pass1_node(i, rp, ci, state, m1, r1, settled);
-}
-
-__device__ __forceinline__ void mis2_pass2_node(int i, const int* __restrict__ rp, const int* __restrict__ ci,
-                                                const int* __restrict__ m1, const int* __restrict__ r1,
-                                                int* __restrict__ state, int* __restrict__ any_undecided) {
-    if (state[i] != kUndecided) return;
-    int mn = 0x7fffffff, root = 0;
-    constexpr int U = 16;  // loads of a batch in flight together
-    const int k0 = rp[i], k1 = rp[i + 1];
-    for (int kb = k0; kb < k1; kb += U) {
-        int jj[U], mj[U], rj[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) jj[u] = kb + u < k1 ? ci[kb + u] : -1;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            mj[u] = jj[u] >= 0 ? m1[jj[u]] : 0x7fffffff;
-            rj[u] = jj[u] >= 0 ? r1[jj[u]] : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            mn = min(mn, mj[u]);
-            root |= rj[u];
-        }
-    }
-    if (root) state[i] = kOut;
-    else if (mn == i) state[i] = kRoot;
-    else *any_undecided = 1;
-}
-
-__global__ void mis2_pass2_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci,
-                                  const int* __restrict__ m1, const int* __restrict__ r1, int* __restrict__ state,
-                                  int* __restrict__ any_undecided) {
-    pdl_wait();
-    pdl_trigger();
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        mis2_pass2_node(i, rp, ci, m1, r1, state, any_undecided);
 }
 
 __global__ void is_root_kernel(int n, const int* __restrict__ state, int* __restrict__ flag) {
@@ -323,30 +345,12 @@ __global__ void attach_kernel(int n, const int* __restrict__ rp, const int* __re
 }
 
 int aggregate_nodes(int n, const int* rp, const int* ci, int* agg, AggWork& w, int* d_count,
-                    int* d_scan_tmp, long scan_tmp_b, cudaStream_t s, int* rounds_out) {
+                    int* d_scan_tmp, long scan_tmp_b, cudaStream_t s) {
     const int threads = 256, blocks = ceil_div(n, threads);
     BAMG_CUDA_TRY(cudaMemsetAsync(w.state, 0, sizeof(int) * (size_t)n, s));
-    if (w.settled) BAMG_CUDA_TRY(cudaMemsetAsync(w.settled, 0, (size_t)n, s));
-    const int batch = 16;
-    const long max_rounds = 4L * n + 64;
-    long rounds = 0;
-    for (;;) {
-        for (int r = 0; r < batch; ++r) {
-            if (r == batch - 1) BAMG_CUDA_TRY(cudaMemsetAsync(w.flag, 0, sizeof(int), s));
-            // agg1 and rootid serve as m1 and r1 during the rounds
-            BAMG_CUDA_TRY(launch_round(mis2_pass1_kernel, blocks, threads, s, n, rp, ci, w.state, w.agg1, w.rootid,
-                                       w.settled));
-            BAMG_CUDA_TRY(launch_round(mis2_pass2_kernel, blocks, threads, s, n, rp, ci, w.agg1, w.rootid, w.state,
-                                       w.flag));
-        }
-        note_launch(2 * batch);
-        rounds += batch;
-        BAMG_CUDA_TRY(cudaMemcpyAsync(w.host_flag, w.flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-        BAMG_CUDA_TRY(cudaStreamSynchronize(s));
-        if (*w.host_flag == 0) break;
-        if (rounds > max_rounds) return BAMG_ETIMEOUT;
-    }
-    if (rounds_out) *rounds_out = (int)rounds;
+    BAMG_CUDA_TRY(cudaMemsetAsync(w.flag, 0, 2 * sizeof(int), s));
+    mis2_kernel<<<chunk_grid(n), kChunk, 0, s>>>(n, rp, ci, w.state, w.flag);
+    note_launch(1);
     // ids = ranks of the roots in ascending index
     is_root_kernel<<<blocks, threads, 0, s>>>(n, w.state, w.rootid);
     int st = exclusive_scan(n, w.rootid, w.rootid, d_scan_tmp, scan_tmp_b, s);
@@ -356,7 +360,9 @@ int aggregate_nodes(int n, const int* rp, const int* ci, int* agg, AggWork& w, i
     note_launch(3);
     BAMG_CUDA_TRY(cudaMemcpyAsync(d_count, w.rootid + n, sizeof(int), cudaMemcpyDeviceToDevice, s));
     BAMG_CUDA_TRY(cudaMemcpyAsync(w.host_flag, d_count, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    BAMG_CUDA_TRY(cudaMemcpyAsync(w.host_flag + 2, w.flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
     BAMG_CUDA_TRY(cudaStreamSynchronize(s));
+    if (w.host_flag[2] != 0) return BAMG_ETIMEOUT;  // a bounded wait ran out
     if (w.host_flag[1] != 0) return BAMG_EINVAL;
     return w.host_flag[0];
 }
@@ -413,69 +419,101 @@ int build_members(int n, int nc, const int* agg, int* agg_ptr, int* members, int
 // ---------------------------------------------------------------------------
 constexpr int kMaxColours = 128;
 
-__device__ __forceinline__ void colour_round_node(int i, const int* __restrict__ rp, const int* __restrict__ ci,
-                                                  int* colour, int* flag) {
-    volatile int* col = colour;
-    if (col[i] >= 0) return;
-    // the row's columns and their colours U at a time: the loads of a batch
-    // are independent (one round trip each instead of one per neighbour)
-    constexpr int U = 16;
-    unsigned long long used0 = 0ull, used1 = 0ull;  // colours 0..63, 64..127
-    const int k0 = rp[i], k1 = rp[i + 1];
-    for (int kb = k0; kb < k1; kb += U) {
-        int jj[U], cj[U];
+// First fit over chunks (see take_chunk): a thread walks the lower entries of
+// its row, notes their colours and stops at the first uncoloured one.  The
+// chunk's own colours are kept in shared memory, where most of the chain of a
+// grid's rows runs.  colour: -1 everywhere on entry; ctl: colour count, failure
+// word (1: a colour of `limit` or more was needed, 2: a wait ran out), ticket.
+__global__ void __launch_bounds__(kChunk) colour_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci,
+                                                        int* colour, int* ctl, int limit) {
+    __shared__ int sc_raw[kChunk];
+    volatile int* sc = sc_raw;
+    constexpr int U = 4;  // entries read together
+    int cmax = -1;
+    for (;;) {
+        const int base = take_chunk(n, ctl + 2, ctl + 1);
+        if (base >= n) break;
+        const int i = base + threadIdx.x;
+        sc[threadIdx.x] = -1;
+        __syncthreads();
+        bool done = i >= n;
+        int k = done ? 0 : rp[i];
+        const int k1 = done ? 0 : rp[i + 1];
+        unsigned long long used[4] = {0ull, 0ull, 0ull, 0ull};
+        for (int spins = 0; __any_sync(0xffffffffu, !done); ++spins) {
+            bool moved = false;
+            if (!done) {
+                int j[U], c[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) jj[u] = kb + u < k1 ? ci[kb + u] : i;
+                for (int u = 0; u < U; ++u) j[u] = k + u < k1 ? ci[k + u] : 0x7fffffff;
 #pragma unroll
-        for (int u = 0; u < U; ++u) cj[u] = jj[u] < i ? col[jj[u]] : 0;
-        bool lower_left = true;
+                for (int u = 0; u < U; ++u)
+                    c[u] = j[u] >= i ? 0 : j[u] >= base ? sc[j[u] - base] : ld_relaxed(colour + j[u]);
+                bool stop = false, end = false;
+                int adv = 0;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (jj[u] >= i) {  // columns ascending: no lower neighbour after this one
-                lower_left = false;
-                continue;
+                for (int u = 0; u < U; ++u) {
+                    stop |= c[u] < 0;
+                    if (!stop && !end) {
+                        if (j[u] >= i) {  // columns ascending: no lower neighbour follows
+                            end = true;
+                        } else {
+#pragma unroll
+                            for (int w = 0; w < 4; ++w)
+                                if ((c[u] >> 6) == w) used[w] |= 1ull << (c[u] & 63);
+                            ++adv;
+                        }
+                    }
+                }
+                k += adv;
+                moved = adv > 0 || end;
+                if (end) {  // the smallest colour not in use
+                    int cc = 256;
+#pragma unroll
+                    for (int w = 3; w >= 0; --w)
+                        if (used[w] != ~0ull) cc = 64 * w + __ffsll((long long)~used[w]) - 1;
+                    if (cc >= limit) {
+                        st_relaxed(ctl + 1, 1);
+                        cc = limit - 1;
+                    }
+                    sc[threadIdx.x] = cc;
+                    st_relaxed(colour + i, cc);
+                    cmax = max(cmax, cc);
+                    done = true;
+                }
             }
-            if (cj[u] < 0) {  // a lower neighbour not coloured yet: next round
-                *flag = 1;
-                return;
+            if (!__any_sync(0xffffffffu, moved)) {
+                if (spins > kChunkSpins) st_relaxed(ctl + 1, 2);
+                if ((spins & 1023) == 1023 && ld_relaxed(ctl + 1) != 0) break;
+                __nanosleep(20);
             }
-            if (cj[u] < 64) used0 |= 1ull << cj[u];
-            else if (cj[u] < kMaxColours) used1 |= 1ull << (cj[u] - 64);
         }
-        if (!lower_left) break;
     }
-    // the smallest colour not in use
-    int c = used0 != ~0ull ? __ffsll((long long)~used0) - 1
-                           : (used1 != ~0ull ? 64 + __ffsll((long long)~used1) - 1 : kMaxColours);
-    if (c >= kMaxColours) {
-        flag[1] = 1;  // too many colours
-        c = kMaxColours - 1;
-    }
-    col[i] = c;
-}
-
-// (programmatic dependent launches as the MIS-2 rounds, over a grid of at
-// most four CTAs per SM: in most rounds most nodes are coloured and return)
-__global__ void colour_round_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci, int* colour,
-                                    int* flag) {
-    pdl_wait();
-    pdl_trigger();
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        colour_round_node(i, rp, ci, colour, flag);
-}
-
-__global__ void max_kernel(int n, const int* __restrict__ v, int* out) {
-    int m = -1;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) m = max(m, v[i]);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+    for (int o = 16; o > 0; o >>= 1) cmax = max(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
+    if ((threadIdx.x & 31) == 0 && cmax >= 0) atomicMax(ctl, cmax + 1);
+}
+
+// *flag = 1 where a stored block (i, j) has no counterpart (j, i); warp per row
+__global__ void asymmetric_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci, int* flag) {
+    const int i = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (i >= n) return;
+    for (int k = rp[i] + (threadIdx.x & 31); k < rp[i + 1]; k += 32) {
+        const int j = ci[k];
+        int lo = rp[j], hi = rp[j + 1];
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (ci[mid] < i) lo = mid + 1;
+            else hi = mid;
+        }
+        if (lo == rp[j + 1] || ci[lo] != i) *flag = 1;
+    }
 }
 
 // Single-CTA Jones-Plassmann for graphs that fit in shared memory: a node is
 // coloured (smallest colour unused by its lower-index neighbours) as soon as
 // its count of uncoloured lower-index neighbours reaches zero; the frontier
-// of such nodes advances one step per iteration.  Same result as the rounds.
+// of such nodes advances one step per iteration.  Same result as colour_kernel.
 // The count of node j is taken from row j and decremented from the rows of
 // its lower neighbours, so the rule needs a structurally symmetric pattern.
 // A pattern that is not symmetric is reported (out[1] = 1), never coloured
@@ -570,11 +608,23 @@ __global__ void __launch_bounds__(1024) colour_worklist_kernel(int n, const int*
     }
 }
 
-// d_flag: 3 device ints, h_flag: 3 pinned host ints
-int colour_nodes(int n, const int* rp, const int* ci, int* colour, int* d_flag, int* h_flag,
-                 cudaStream_t s, int* n_colours, int* rounds_out, int* d_queue) {
-    const int threads = 256, blocks = ceil_div(n, threads), rgrid = round_grid(n, threads);
-    if (n <= kWorklistMaxNodes && d_queue) {
+// d_flag: 4 device ints, h_flag: 4 pinned host ints, d_queue: 2n ints of scratch
+int colour_nodes(int n, const int* rp, const int* ci, int* colour, int* d_flag, int* h_flag, cudaStream_t s,
+                 int* n_colours, int* d_queue) {
+    // Graphs of up to kWorklistMaxNodes nodes may use 255 colours and must be
+    // structurally symmetric: one that is not goes to colour_worklist_kernel,
+    // whose counts of uncoloured neighbours report it.  (That kernel, one CTA,
+    // took 1.5 ms for 129^2 nodes.)  Larger graphs may use kMaxColours.
+    const bool small = n <= kWorklistMaxNodes;
+    BAMG_CUDA_TRY(cudaMemsetAsync(colour, 0xff, sizeof(int) * (size_t)n, s));
+    BAMG_CUDA_TRY(cudaMemsetAsync(d_flag, 0, 4 * sizeof(int), s));
+    colour_kernel<<<chunk_grid(n), kChunk, 0, s>>>(n, rp, ci, colour, d_flag, small ? 255 : kMaxColours);
+    if (small) asymmetric_kernel<<<ceil_div((long)n * 32, 256), 256, 0, s>>>(n, rp, ci, d_flag + 3);
+    note_launch(small ? 2 : 1);
+    BAMG_CUDA_TRY(cudaMemcpyAsync(h_flag, d_flag, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    BAMG_CUDA_TRY(cudaStreamSynchronize(s));
+    if (h_flag[1] == 2) return BAMG_ETIMEOUT;
+    if (small && h_flag[3]) {
         const size_t smem = (size_t)n * 5 + 16;
         // the limit is always raised to what the largest accepted graph needs,
         // never to this call's size: amg_colour_noalloc launches the same
@@ -586,67 +636,63 @@ int colour_nodes(int n, const int* rp, const int* ci, int* colour, int* d_flag, 
         note_launch(1);
         BAMG_CUDA_TRY(cudaMemcpyAsync(h_flag, d_flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
         BAMG_CUDA_TRY(cudaStreamSynchronize(s));
-        if (h_flag[1]) return BAMG_EUNSUPPORTED;
-        *n_colours = h_flag[0];
-        if (rounds_out) *rounds_out = 0;
-        return BAMG_OK;
     }
-    BAMG_CUDA_TRY(cudaMemsetAsync(colour, 0xff, sizeof(int) * (size_t)n, s));
-    BAMG_CUDA_TRY(cudaMemsetAsync(d_flag, 0, 3 * sizeof(int), s));
-    const int batch = 32;
-    const long max_rounds = 2L * n + 64;
-    long rounds = 0;
-    for (;;) {
-        for (int r = 0; r < batch; ++r) {
-            if (r == batch - 1) BAMG_CUDA_TRY(cudaMemsetAsync(d_flag, 0, sizeof(int), s));
-            BAMG_CUDA_TRY(launch_round(colour_round_kernel, rgrid, threads, s, n, rp, ci, colour, d_flag));
-        }
-        note_launch(batch);
-        rounds += batch;
-        BAMG_CUDA_TRY(cudaMemcpyAsync(h_flag, d_flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-        BAMG_CUDA_TRY(cudaStreamSynchronize(s));
-        if (h_flag[1]) return BAMG_EUNSUPPORTED;
-        if (h_flag[0] == 0) break;
-        if (rounds > max_rounds) return BAMG_ETIMEOUT;
-    }
-    if (rounds_out) *rounds_out = (int)rounds;
-    BAMG_CUDA_TRY(cudaMemsetAsync(d_flag + 2, 0xff, sizeof(int), s));
-    max_kernel<<<min(ceil_div(n, 256), 1024), 256, 0, s>>>(n, colour, d_flag + 2);
-    note_launch(1);
-    BAMG_CUDA_TRY(cudaMemcpyAsync(h_flag + 2, d_flag + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BAMG_CUDA_TRY(cudaStreamSynchronize(s));
-    *n_colours = h_flag[2] + 1;
+    if (h_flag[1]) return BAMG_EUNSUPPORTED;
+    *n_colours = h_flag[0];
     return BAMG_OK;
 }
 
-// nodes ordered by (colour, index): one stable compaction per colour
-__global__ void eq_flag_kernel(int n, const int* __restrict__ v, int c, int* __restrict__ flag) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = v[i] == c ? 1 : 0;
+// Nodes ordered by (colour, index): a counting sort over tiles of kChunk nodes.
+// count[c * tiles + t] = nodes of colour c in tile t; their exclusive scan is
+// the first place of every (colour, tile), and a node's place follows from the
+// lower nodes of its colour in its tile.  (One stable compaction per colour,
+// six launches each, took 0.2 ms a level.)
+__global__ void __launch_bounds__(kChunk) colour_count_kernel(int n, int C, int tiles, const int* __restrict__ colour,
+                                                              int* __restrict__ count) {
+    extern __shared__ int hist[];  // C
+    for (int c = threadIdx.x; c < C; c += kChunk) hist[c] = 0;
+    __syncthreads();
+    const int i = blockIdx.x * kChunk + threadIdx.x;
+    if (i < n) atomicAdd(hist + colour[i], 1);
+    __syncthreads();
+    for (int c = threadIdx.x; c < C; c += kChunk) count[(size_t)c * tiles + blockIdx.x] = hist[c];
 }
-__global__ void compact_kernel(int n, const int* __restrict__ v, int c, const int* __restrict__ pos,
-                               const int* __restrict__ base, int* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && v[i] == c) out[*base + pos[i]] = i;
-}
-__global__ void advance_kernel(int* __restrict__ colour_ptr, int c, const int* __restrict__ pos, int n) {
-    colour_ptr[c + 1] = colour_ptr[c] + pos[n];
+__global__ void __launch_bounds__(kChunk) colour_place_kernel(int n, int C, int tiles, const int* __restrict__ colour,
+                                                              const int* __restrict__ first, int* __restrict__ nodes,
+                                                              int* __restrict__ colour_ptr) {
+    extern __shared__ int hist[];  // [warps][C]: nodes of every colour in each warp
+    constexpr int W = kChunk / 32;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int e = threadIdx.x; e < W * C; e += kChunk) hist[e] = 0;
+    __syncthreads();
+    const int i = blockIdx.x * kChunk + threadIdx.x;
+    const int c = i < n ? colour[i] : -1;
+    const unsigned same = __match_any_sync(0xffffffffu, c);
+    const int rank = __popc(same & ((1u << lane) - 1u));
+    if (c >= 0 && rank == 0) hist[w * C + c] = __popc(same);
+    __syncthreads();
+    if (c >= 0) {
+        int p = first[(size_t)c * tiles + blockIdx.x] + rank;
+        for (int v = 0; v < w; ++v) p += hist[v * C + c];
+        nodes[p] = i;
+    }
+    if (blockIdx.x == 0)
+        for (int q = threadIdx.x; q <= C; q += kChunk) colour_ptr[q] = first[(size_t)q * tiles];
 }
 
-// d_tmp: n + 1 + scan tmp ints
-int colour_order(int n, int C, const int* colour, int* colour_ptr, int* nodes, int* d_tmp,
-                 cudaStream_t s) {
-    int* pos = d_tmp;
-    int* scan_tmp = d_tmp + n + 1;
-    BAMG_CUDA_TRY(cudaMemsetAsync(colour_ptr, 0, sizeof(int), s));
-    for (int c = 0; c < C; ++c) {
-        eq_flag_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, colour, c, pos);
-        int st = exclusive_scan(n, pos, pos, scan_tmp, scan_tmp_bytes(n), s);
-        if (st) return st;
-        compact_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, colour, c, pos, colour_ptr + c, nodes);
-        advance_kernel<<<1, 1, 0, s>>>(colour_ptr, c, pos, n);
-    }
-    return launched(3 * C);
+// ints of scratch for colour_order
+long colour_order_ints(int n, int C) {
+    const long m = (long)C * ceil_div(n, kChunk);
+    return m + 1 + scan_tmp_bytes((int)m) / (long)sizeof(int) + 16;
+}
+int colour_order(int n, int C, const int* colour, int* colour_ptr, int* nodes, int* d_tmp, cudaStream_t s) {
+    const int tiles = ceil_div(n, kChunk), m = C * tiles;
+    colour_count_kernel<<<tiles, kChunk, sizeof(int) * C, s>>>(n, C, tiles, colour, d_tmp);
+    const int st = exclusive_scan(m, d_tmp, d_tmp, d_tmp + m + 1, scan_tmp_bytes(m), s);
+    if (st) return st;
+    colour_place_kernel<<<tiles, kChunk, sizeof(int) * C * (kChunk / 32), s>>>(n, C, tiles, colour, d_tmp, nodes,
+                                                                               colour_ptr);
+    return launched(2);
 }
 
 // ---------------------------------------------------------------------------
@@ -737,35 +783,90 @@ int rap_fill_cols(int nc, const int* rp_c, const int* tmp_cols, int cap, int* ci
     return launched(1);
 }
 
+// The warp takes a member's blocks 32 at a time: each lane finds the place of
+// its block in the coarse row (the loads and searches of 32 blocks together),
+// then the blocks are added one after another.  Rows of up to kRapSmem bytes
+// are accumulated in shared memory, longer ones in place: block after block
+// added to global memory is a chain of 700 round trips for a row of the 3D
+// grid (1.4 ms; 0.4 ms this way, 65^3 nodes; FP64 floor 0.19 ms).
+constexpr int kRapSmem = 8192;
 __global__ void __launch_bounds__(kRapWarps * 32)
     rap_numeric_kernel(int b, int nc, const int* __restrict__ agg_ptr, const int* __restrict__ members,
                        const int* __restrict__ rp, const int* __restrict__ ci,
                        const double* __restrict__ vals, const int* __restrict__ agg,
                        const int* __restrict__ rp_c, const int* __restrict__ ci_c,
                        double* __restrict__ vals_c) {
+    __shared__ double sh[kRapWarps][kRapSmem / 8];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int I = blockIdx.x * kRapWarps + wid;
     if (I >= nc) return;
     const int bb = b * b;
-    const int c0 = rp_c[I], c1 = rp_c[I + 1];
+    const int c0 = rp_c[I], c1 = rp_c[I + 1], ne = (c1 - c0) * bb;
     double* out = vals_c + (size_t)c0 * bb;
-    for (int e = lane; e < (c1 - c0) * bb; e += 32) out[e] = 0.0;
+    const bool local = ne <= kRapSmem / 8;
+    double* acc = local ? sh[wid] : out;
+    for (int e = lane; e < ne; e += 32) acc[e] = 0.0;
     __syncwarp();
     for (int q = agg_ptr[I]; q < agg_ptr[I + 1]; ++q) {
         const int i = members[q];
-        for (int k = rp[i]; k < rp[i + 1]; ++k) {
-            const int J = agg[ci[k]];
-            int lo = c0, hi = c1;  // binary search of J in the sorted coarse row
-            while (lo < hi) {
-                int m = (lo + hi) >> 1;
-                if (ci_c[m] < J) lo = m + 1;
-                else hi = m;
+        const int k0 = rp[i], k1 = rp[i + 1];
+        for (int kb = k0; kb < k1; kb += 32) {
+            int at = 0;
+            if (kb + lane < k1) {
+                const int J = agg[ci[kb + lane]];
+                int lo = c0, hi = c1;  // binary search of J in the sorted coarse row
+                while (lo < hi) {
+                    const int m = (lo + hi) >> 1;
+                    if (ci_c[m] < J) lo = m + 1;
+                    else hi = m;
+                }
+                at = (lo - c0) * bb;
             }
-            double* dst = vals_c + (size_t)lo * bb;
-            const double* src = vals + (size_t)k * bb;
-            for (int e = lane; e < bb; e += 32) dst[e] = __dadd_rn(dst[e], src[e]);
+            const int cnt = min(32, k1 - kb);
+            const double* src = vals + (size_t)kb * bb;
+            // two blocks side by side when both fit the warp (b <= 4), else one:
+            // either way an entry's additions keep the order of the blocks
+            if (bb <= 16) {
+                constexpr int U = 4;  // pairs loaded together
+                const int half = lane >> 4, e = lane & 15;
+                for (int t = 0; t < cnt; t += 2 * U) {
+                    double v[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int tb = t + 2 * u + half;
+                        v[u] = tb < cnt && e < bb ? src[(size_t)tb * bb + e] : 0.0;
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int t0 = t + 2 * u;
+                        const int d0 = __shfl_sync(0xffffffffu, at, t0 & 31);
+                        const int d1 = __shfl_sync(0xffffffffu, at, (t0 + 1) & 31);
+                        const bool on = t0 + half < cnt && e < bb;
+                        const int d = (half ? d1 : d0) + e;
+                        if (d0 != d1) {  // two places: both at once
+                            if (on) acc[d] = __dadd_rn(acc[d], v[u]);
+                        } else {
+                            if (on && half == 0) acc[d] = __dadd_rn(acc[d], v[u]);
+                            __syncwarp();
+                            if (on && half == 1) acc[d] = __dadd_rn(acc[d], v[u]);
+                        }
+                        __syncwarp();
+                    }
+                }
+            } else {
+                for (int t = 0; t < cnt; ++t) {
+                    const int d = __shfl_sync(0xffffffffu, at, t);
+                    const double v0 = lane < bb ? src[(size_t)t * bb + lane] : 0.0;
+                    const double v1 = lane + 32 < bb ? src[(size_t)t * bb + lane + 32] : 0.0;
+                    if (lane < bb) acc[d + lane] = __dadd_rn(acc[d + lane], v0);
+                    if (lane + 32 < bb) acc[d + lane + 32] = __dadd_rn(acc[d + lane + 32], v1);
+                }
+            }
         }
     }
+    __syncwarp();
+    if (local)
+        for (int e = lane; e < ne; e += 32) out[e] = acc[e];
 }
 
 int rap_numeric(int b, int nc, const int* agg_ptr, const int* members, const int* rp, const int* ci,
