@@ -264,8 +264,8 @@ struct bamg_ctx {
         int status = BAMG_OK, n_colours = 0;
         int *flag = nullptr, *queue = nullptr, *pin = nullptr;
     } cjob[kMaxLevels];
-    // the tensor-core coarsest LU enqueued on cap_stream ahead of the smoother
-    // data of the finer levels (no host synchronisation inside it); its own
+    // the coarsest LU enqueued on cap_stream ahead of the smoother data of the
+    // finer levels (no host synchronisation inside it); its own
     // error word, its temporaries released once the setup stream has joined it
     bool coarse_pending = false;
     cudaEvent_t coarse_ev = nullptr;
@@ -1234,27 +1234,38 @@ static int colour_join(bamg_ctx* h, int l, Level& L, cudaStream_t s, bool* done)
     return BAMG_OK;
 }
 
-// The tensor-core coarsest LU and inverse of a single system (FP32 coarsest
-// solve of 224 to 2048 unknowns) enqueued on cap_stream, where it runs while
-// the setup stream builds the finer levels' smoother data; the coarse branch
-// of setup_impl joins it.  (The CUDA-core paths keep their place: their
-// cooperative kernels want every CTA resident at once.)
+// The coarsest LU and inverse of a single system enqueued on cap_stream, where
+// it runs while the setup stream colours the finer levels and builds their
+// smoother data; the coarse branch of setup_impl joins it.  The tensor-core path
+// (FP32, 224 to 2048 unknowns) and the cluster path (small matrices) go ahead
+// like this: neither synchronises the host.  (The other CUDA-core paths keep
+// their place: their cooperative kernels want every CTA resident at once.)
 static int coarse_begin(bamg_ctx* h, cudaStream_t s) {
-    if (h->nsys > 1 || h->p.coarse_prec != 32 || h->p.coarse_tc != 1) return BAMG_OK;
+    if (h->nsys > 1) return BAMG_OK;
     const Level& L = h->lev[h->nlev - 1];
     const long nd = (long)L.n * h->b;
-    if (nd > kMaxCoarseDense || nd <= kCoarseTcMin || !tc_lu_supported((int)nd)) return BAMG_OK;
+    const bool f32 = h->p.coarse_prec == 32;
+    const bool tc = f32 && h->p.coarse_tc == 1 && nd > kCoarseTcMin && nd <= kMaxCoarseDense && tc_lu_supported((int)nd);
+    if (!tc && !lu_in_cluster(nd, f32)) return BAMG_OK;
     h->nd = (int)nd;
-    h->coarse_tc_used = true;
+    h->coarse_tc_used = tc;
     TRY(h->alloc(&h->coarse_a, (size_t)(nd * nd)));
     TRY(h->alloc(&h->coarse_piv, (size_t)nd));
-    TRY(h->alloc(&h->coarse_inv32, (size_t)(nd * nd)));
     TRY(h->alloc(&h->coarse_err, 4));
     float *a32 = nullptr, *lt32 = nullptr, *work32 = nullptr;
-    TRY(h->alloc(&a32, (size_t)(nd * nd)));
-    TRY(h->alloc(&lt32, (size_t)(nd * nd)));
-    TRY(h->alloc(&work32, (size_t)tc_lu_scratch_floats((int)nd)));
-    h->coarse_tmp = {a32, lt32, work32};
+    double *lt64 = nullptr, *work64 = nullptr;
+    if (f32) {
+        TRY(h->alloc(&h->coarse_inv32, (size_t)(nd * nd)));
+        TRY(h->alloc(&a32, (size_t)(nd * nd)));
+        TRY(h->alloc(&lt32, (size_t)(nd * nd)));
+    } else {
+        TRY(h->alloc(&h->coarse_inv, (size_t)(nd * nd)));
+        TRY(h->alloc(&lt64, (size_t)(nd * nd)));
+    }
+    if (tc) TRY(h->alloc(&work32, (size_t)tc_lu_scratch_floats((int)nd)));
+    else TRY(h->alloc(&work64, (size_t)dense_lu_scratch((int)nd)));
+    for (void* q : {(void*)a32, (void*)lt32, (void*)work32, (void*)lt64, (void*)work64})
+        if (q) h->coarse_tmp.push_back(q);
     BAMG_CUDA_TRY(cudaMemsetAsync(h->coarse_err, 0, 4 * sizeof(int), s));
     BAMG_CUDA_TRY(cudaEventCreateWithFlags(&h->coarse_ev, cudaEventDisableTiming));
     BAMG_CUDA_TRY(cudaEventRecord(h->coarse_ev, s));  // the coarsest values and the allocations above
@@ -1262,8 +1273,13 @@ static int coarse_begin(bamg_ctx* h, cudaStream_t s) {
     BAMG_CUDA_TRY(cudaStreamWaitEvent(cs, h->coarse_ev, 0));
     h->coarse_pending = true;
     TRY(coarse_dense(h->b, L.n, L.rp, L.ci, L.vals64, h->coarse_a, cs));
-    TRY(launch_convert_d2f(nd * nd, h->coarse_a, a32, cs));
-    TRY(dense_lu_inverse_tc((int)nd, a32, h->coarse_piv, h->coarse_inv32, lt32, work32, h->coarse_err, cs));
+    if (f32) TRY(launch_convert_d2f(nd * nd, h->coarse_a, a32, cs));
+    if (tc) TRY(dense_lu_inverse_tc((int)nd, a32, h->coarse_piv, h->coarse_inv32, lt32, work32, h->coarse_err, cs));
+    else if (f32)
+        TRY(dense_lu_inverse<float>((int)nd, a32, h->coarse_piv, h->coarse_inv32, lt32, work64, h->coarse_err, cs));
+    else
+        TRY(dense_lu_inverse<double>((int)nd, h->coarse_a, h->coarse_piv, h->coarse_inv, lt64, work64, h->coarse_err,
+                                     cs));
     BAMG_CUDA_TRY(cudaEventRecord(h->coarse_ev, cs));
     return BAMG_OK;
 }
@@ -1607,7 +1623,7 @@ static int setup_impl(bamg_ctx* h, const int* row_ptr, const int* col_idx, const
         h->t_phase[5] += ms_since(tp);
         tp = Clock::now();
     } else if (h->coarse_pending) {
-        // the tensor-core LU enqueued by coarse_begin
+        // the LU enqueued by coarse_begin
         BAMG_CUDA_TRY(cudaStreamWaitEvent(s, h->coarse_ev, 0));
         h->coarse_pending = false;
         BAMG_CUDA_TRY(cudaMemcpyAsync(h->h_pin, h->coarse_err, sizeof(int), cudaMemcpyDeviceToHost, s));

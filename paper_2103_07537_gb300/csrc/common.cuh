@@ -560,6 +560,8 @@ int coarse_dense(int b, int n, const int* rp, const int* ci, const double* vals,
 // receives A^{-1}; piv (nd ints) receives the logical row position of every
 // row; lt: nd*nd T of scratch; work: dense_lu_scratch(nd) doubles of scratch
 long dense_lu_scratch(int nd);
+// (matrices that the cluster LU takes: no cooperative launch)
+bool lu_in_cluster(long nd, bool fp32);
 template <typename T>
 int dense_lu_inverse(int nd, T* a, int* piv, T* inv, T* lt, double* work, int* err, cudaStream_t s);
 
@@ -569,7 +571,7 @@ int dense_lu_inverse(int nd, T* a, int* piv, T* inv, T* lt, double* work, int* e
 // pivoting; x: nd*nd floats of scratch, work: tc_lu_scratch_floats(nd)
 // floats.  A pivot below 1e-9 ||a||_inf sets kDevSingularCoarse, a bounded
 // wait that ran out kDevTimeout (in *err).
-constexpr int kCoarseTcMin = 223;  // smaller coarsest matrices: the one-CTA shared-memory LU
+constexpr int kCoarseTcMin = 223;  // smaller coarsest matrices: the cluster LU
 bool tc_lu_supported(int nd);
 long tc_lu_scratch_floats(int nd);
 int dense_lu_inverse_tc(int nd, float* a, int* pos, float* inv, float* x, float* work, int* err, cudaStream_t s);

@@ -10,7 +10,11 @@
 // node that could influence it has decided), so the result does not depend
 // on thread scheduling.  A state only ever moves from "undecided" to a final
 // value, so a stale read can only delay a decision.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace bamg {
 
@@ -993,7 +997,7 @@ int coarse_dense(int b, int n, const int* rp, const int* ci, const double* vals,
     return launched(1);
 }
 
-// LU factorisation.  Small nd: one CTA factors the matrix held in shared
+// LU factorisation.  Small nd: one cluster holds the matrix in its shared
 // memory; larger: one cooperative launch (below), else one pivot kernel and
 // one rank-1 update kernel per column.  All perform the same rounded
 // operations in the same order per entry, so the factors do not depend on
@@ -1001,10 +1005,12 @@ int coarse_dense(int b, int n, const int* rp, const int* ci, const double* vals,
 // factors the FP32 copy of the coarsest matrix for FP32 cycles (GB300 issues
 // FP32 at 64 times its FP64 rate).
 constexpr int kLuThreads = 1024;
-// largest nd whose nd^2 entries fit 199.7 KB of shared memory (158^2 doubles)
+// largest nd of the cluster LU (FP64: 16 CTAs of at most 220 KB hold 600^2;
+// FP32: the tensor-core or blocked paths follow)
+constexpr int kClusterLuThreads = 512;
 template <typename T>
-struct LuSmem {
-    static constexpr int kMax = sizeof(T) == 8 ? 158 : 223;
+struct ClusterLu {
+    static constexpr int kMax = sizeof(T) == 8 ? 600 : 223;
 };
 // a smallest pivot of 1e-14 (FP64) or 1e-9 (FP32) times the infinity norm
 // marks the matrix singular.  (In FP32 pivots between that and the rounding
@@ -1068,64 +1074,134 @@ __device__ __forceinline__ void pivot_search(const T* a, int nd, int k, T* red_v
     __syncthreads();
 }
 
-// infinity norm (largest absolute row sum) of the nd x nd matrix a
+// Small matrices: one thread-block cluster of C CTAs, column j of the matrix in
+// the shared memory of CTA j % C (column by column).  For column k its owner
+// finds the pivot and sends it with the multipliers to every CTA (distributed
+// shared memory), one cluster barrier, then each CTA swaps the two rows in its
+// columns and updates those right of k, a warp per column.  The multipliers
+// alternate between two buffers: the owner of column k + 1 may send while
+// others still read those of k, and the barrier of k + 1 comes between the
+// readers of k and the writer of k + 2.  Bound by the chain of nd steps (pivot,
+// division, barrier: about 1.2 us) and by FP64 (a product and a difference per
+// entry, two a clock per SM: one CTA alone took 1.78 ms for nd = 150).
 template <typename T>
-__device__ __forceinline__ T inf_norm(const T* a, int nd, T* red_v) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    T m = T(0);
-    for (int r = tid; r < nd; r += blockDim.x) {
-        T sum = T(0);
-        for (int c = 0; c < nd; ++c) sum += fabs(a[(size_t)r * nd + c]);
-        m = fmax(m, sum);
+__global__ void __launch_bounds__(kClusterLuThreads) lu_cluster_kernel(int nd, T* __restrict__ g, const T* __restrict__ norm,
+                                                                       int* __restrict__ piv, int* err) {
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int ncl = (nd - rank + C - 1) / C;  // own columns
+    extern __shared__ __align__(16) unsigned char lu_sh[];
+    T* mult = reinterpret_cast<T*>(lu_sh);  // [2][nd]
+    T* sa = mult + 2 * nd;                  // [ncl][nd]
+    __shared__ int s_pivot[2], s_p;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
+    for (int r = w; r < nd; r += nw)
+        for (int l = lane; l < ncl; l += 32) sa[(size_t)l * nd + r] = g[(size_t)r * nd + l * C + rank];
+    cl.sync();  // every CTA is there before the first remote store
+    const T tiny = lu_tiny<T>() * norm[0];
+    bool singular = norm[0] == T(0);
+    for (int k = 0; k < nd; ++k) {
+        const int slot = k & 1;
+        if (k % C == rank) {  // whole CTA
+            T* col = sa + (size_t)(k / C) * nd;
+            if (w == 0) {  // first row >= k of maximal |a|
+                T best = T(-1);
+                int bi = nd;
+                for (int r = k + lane; r < nd; r += 32) {
+                    const T v = fabs(col[r]);
+                    if (v > best) {
+                        best = v;
+                        bi = r;
+                    }
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const T ov = __shfl_xor_sync(0xffffffffu, best, o);
+                    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+                    if (ov > best || (ov == best && oi < bi)) {
+                        best = ov;
+                        bi = oi;
+                    }
+                }
+                if (!(best >= tiny)) singular = true;
+                bi = min(bi, nd - 1);  // (NaN: no row compares)
+                __syncwarp();  // every lane's reads before the swap
+                if (lane == 0) {
+                    const T t = col[k];
+                    col[k] = col[bi];
+                    col[bi] = t;
+                    s_p = bi;
+                    piv[k] = bi;
+                }
+            }
+            __syncthreads();
+            const int p = s_p;
+            const T akk = col[k];
+            for (int r = k + 1 + tid; r < nd; r += blockDim.x) {
+                const T m = rn_div(col[r], akk);
+                col[r] = m;
+                for (int c = 0; c < C; ++c) cl.map_shared_rank(mult, c)[slot * nd + r] = m;
+            }
+            if (tid < C) *cl.map_shared_rank(s_pivot + slot, tid) = p;
+        }
+        cl.sync();
+        const int p = s_pivot[slot];
+        const T* m = mult + slot * nd;
+        for (int l = w; l < ncl; l += nw) {
+            const int j = l * C + rank;
+            if (j == k) continue;
+            T* col = sa + (size_t)l * nd;
+            if (p != k) {
+                if (lane == 0) {
+                    const T t = col[k];
+                    col[k] = col[p];
+                    col[p] = t;
+                }
+                __syncwarp();
+            }
+            if (j < k) continue;
+            const T akj = col[k];
+            for (int r = k + 1 + lane; r < nd; r += 32) col[r] = rn_sub(col[r], rn_mul(m[r], akj));
+        }
+        __syncthreads();  // the next column's owner searches it with its first warp
     }
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) red_v[wid] = m;
-    __syncthreads();
-    T mm = T(0);
-    for (int w = 0; w < (int)(blockDim.x / 32); ++w) mm = fmax(mm, red_v[w]);
-    __syncthreads();
-    return mm;
+    if (singular) set_error(err, kDevSingularCoarse);
+    for (int r = w; r < nd; r += nw)
+        for (int l = lane; l < ncl; l += 32) g[(size_t)r * nd + l * C + rank] = sa[(size_t)l * nd + r];
+    cl.sync();  // no CTA leaves while another may still write to it
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kLuThreads) lu_smem_kernel(int nd, T* __restrict__ g, int* __restrict__ piv,
-                                                             int* err) {
-    extern __shared__ __align__(16) unsigned char lu_sh[];
-    T* sa = reinterpret_cast<T*>(lu_sh);
-    __shared__ T red_v[kLuThreads / 32];
-    __shared__ int red_i[kLuThreads / 32];
-    __shared__ T col[LuSmem<T>::kMax];
-    const int tid = threadIdx.x;
-    for (int e = tid; e < nd * nd; e += blockDim.x) sa[e] = g[e];
-    __syncthreads();
-    const T norm = inf_norm(sa, nd, red_v);
-    bool singular = norm == T(0);
-    for (int k = 0; k < nd; ++k) {
-        T best;
-        int p;
-        pivot_search(sa, nd, k, red_v, red_i, &best, &p);
-        if (!(best >= lu_tiny<T>() * norm)) singular = true;
-        if (tid == 0) piv[k] = p;
-        if (p != k)
-            for (int c = tid; c < nd; c += blockDim.x) {
-                const T t = sa[k * nd + c];
-                sa[k * nd + c] = sa[p * nd + c];
-                sa[p * nd + c] = t;
-            }
-        __syncthreads();
-        const T akk = sa[k * nd + k];
-        for (int r = k + 1 + tid; r < nd; r += blockDim.x) col[r] = rn_div(sa[r * nd + k], akk);
-        __syncthreads();
-        const int m = nd - k - 1;
-        for (int e = tid; e < m * m; e += blockDim.x) {
-            const int r = k + 1 + e / m, c = k + 1 + e % m;
-            sa[r * nd + c] = rn_sub(sa[r * nd + c], rn_mul(col[r], sa[k * nd + c]));
-        }
-        for (int r = k + 1 + tid; r < nd; r += blockDim.x) sa[r * nd + k] = col[r];
-        __syncthreads();
-    }
-    if (singular && tid == 0) set_error(err, kDevSingularCoarse);
-    for (int e = tid; e < nd * nd; e += blockDim.x) g[e] = sa[e];
+static size_t cluster_lu_smem(int nd, int C) {
+    return sizeof(T) * (size_t)nd * (2 + (nd + C - 1) / C);
+}
+// CTAs of the cluster for nd unknowns (0: another path)
+template <typename T>
+static int cluster_lu_size(int nd) {
+    if (nd > ClusterLu<T>::kMax) return 0;
+    return nd <= 256 ? 8 : 16;
+}
+bool lu_in_cluster(long nd, bool fp32) {
+    return nd <= (fp32 ? ClusterLu<float>::kMax : ClusterLu<double>::kMax);
+}
+template <typename T>
+static cudaError_t launch_cluster_lu(int nd, int C, T* a, const T* norm, int* piv, int* err, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3((unsigned)C);
+    cfg.blockDim = dim3(kClusterLuThreads);
+    cfg.dynamicSmemBytes = cluster_lu_smem<T>(nd, C);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaFuncSetAttribute(lu_cluster_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)cfg.dynamicSmemBytes);
+    if (e == cudaSuccess && C > 8)
+        e = cudaFuncSetAttribute(lu_cluster_kernel<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, lu_cluster_kernel<T>, nd, a, norm, piv, err) : e;
 }
 
 // infinity norm over the grid: one warp per row (coalesced), the row maxima
@@ -1850,15 +1926,14 @@ int dense_lu_inverse(int nd, T* a, int* piv, T* inv, T* lt, double* work, int* e
                           cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
                           sms <= kCoopMaxCtas;
     if (!can_coop) cudaGetLastError();
-    if (nd <= LuSmem<T>::kMax) {
-        const size_t smem = sizeof(T) * (size_t)nd * nd;
-        BAMG_CUDA_TRY(cudaFuncSetAttribute(lu_smem_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        lu_smem_kernel<T><<<1, kLuThreads, smem, s>>>(nd, a, piv, err);
+    BAMG_CUDA_TRY(cudaMemsetAsync(col + nd, 0, sizeof(T), s));
+    lu_norm_rows_kernel<T><<<ceil_div((long)nd * 32, 256), 256, 0, s>>>(nd, a, col + nd);
+    n += 1;
+    const int cluster = cluster_lu_size<T>(nd);
+    if (cluster > 0 && launch_cluster_lu<T>(nd, cluster, a, col + nd, piv, err, s) == cudaSuccess) {
         n += 1;
     } else {
-        BAMG_CUDA_TRY(cudaMemsetAsync(col + nd, 0, sizeof(T), s));
-        lu_norm_rows_kernel<T><<<ceil_div((long)nd * 32, 256), 256, 0, s>>>(nd, a, col + nd);
-        n += 1;
+        (void)cudaGetLastError();
         int per_sm = 0;
         size_t smem = 0;
         // FP32: blocked, with the owned rows resident in shared memory, when
