@@ -151,35 +151,10 @@ __device__ __forceinline__ void stage_params(const uint16_t* __restrict__ p16, f
     __syncthreads();
 }
 
-// forward pass of one training row: xh, and h1, h2 into shared-memory rows
-__device__ __forceinline__ void row_forward(const float* __restrict__ sp, const float* __restrict__ x, float* xh,
-                                            float* h1, float* h2, float* y) {
-#pragma unroll
-    for (int m = 0; m < kNF; ++m) xh[m] = (x[m] - sp[kOXM + m]) * sp[kOXS + m];
-    for (int k = 0; k < kNH; ++k) {
-        float a = 0.f;
-#pragma unroll
-        for (int m = 0; m < kNF; ++m) a = fmaf(sp[kOW1 + k * kNF + m], xh[m], a);
-        h1[k] = tanhf(a + sp[kOB1 + k]);
-    }
-    float y0 = 0.f, y1 = 0.f;
-    for (int j = 0; j < kNH; ++j) {
-        float a = 0.f;
-#pragma unroll
-        for (int k = 0; k < kNH; ++k) a = fmaf(sp[kOW2 + j * kNH + k], h1[k], a);
-        const float h = tanhf(a + sp[kOB2 + j]);
-        h2[j] = h;
-        y0 = fmaf(sp[kOW3 + j], h, y0);
-        y1 = fmaf(sp[kOW3 + kNH + j], h, y1);
-    }
-    y[0] = y0 + sp[kOB3];
-    y[1] = y1 + sp[kOB3 + 1];
-}
-
-// The same arithmetic as row_forward (every sum from 0 in ascending index
-// order, bias added last) with the loops exchanged: h1[k] is produced one at
-// a time and folded into the 64 accumulators of the second layer at once, so
-// no activation array is indexed at run time and nothing spills.
+// One row (every sum from 0 in ascending index order, bias added last): h1[k]
+// is produced one at a time and folded into the 64 accumulators of the second
+// layer at once, so no activation array is indexed at run time and nothing
+// spills.
 __device__ __forceinline__ void row_infer(const float* __restrict__ sp, const float* __restrict__ x, float* y) {
     float xh[kNF], a2[kNH];
 #pragma unroll
@@ -232,135 +207,226 @@ int launch_pack_half(const float* p, uint16_t* p16, cudaStream_t s) {
     return launched(1);
 }
 
-// Gradient of the mean squared error over one tile of kTileRows rows.
-// Phase 1, thread per row: forward, dL/dy, back through both tanh layers;
-// the activations and pre-activation gradients of the tile go to shared
-// memory.  Phase 2, all threads: the parameter gradients of the tile as
-// sums over its rows in ascending order, written to partial[tile][NTRAIN].
-constexpr int kTileRows = 64;
+// Gradient of the mean squared error.  A CTA takes tiles of kTileRows rows
+// (tile = its index, then every grid-th one).  Phase 1, eight threads per row
+// (thread g the hidden units g, g + 8, ...): forward, dL/dy, back through both
+// tanh layers; the activations and pre-activation gradients of the tile go to
+// shared memory, row strides padded so that the eight units a row reads at
+// once lie in distinct banks.  Phase 2: every thread adds the tile's rows, in
+// ascending order, to its own parameter gradients in registers (a 4 x 4 patch
+// of W2), written to partial[CTA][NTRAIN] after the last tile.  The partials
+// are added in CTA order by grad_reduce_kernel: the sum depends on n alone.
+// Latency-bound at the training batch of 4096 rows (128 tiles): one thread per
+// row and one output per thread took 45 us, and the reduction, one thread per
+// output over all tiles, 12 us.
+constexpr int kTileRows = 32;
 constexpr int kGradThreads = 256;
-constexpr int kLd = kNH + 1;  // padded row stride of the activation tiles
+constexpr int kGradCtas = 304;  // at most two per SM
+constexpr int kLd = kNH + 1;    // padded row stride
+constexpr int kUnits = 8;       // hidden units of a thread
 
 struct GradSmem {
-    float sp[BAMG_MLP_NPARAMS];
+    float w1[kNH][kNF + 1];
+    float w2[kNH][kLd];
+    float b1[kNH], b2[kNH], w3[kNO][kNH], b3[kNO], xm[kNF], xs[kNF];
     float h1[kTileRows][kLd];
     float h2[kTileRows][kLd];
     float da1[kTileRows][kLd];
     float da2[kTileRows][kLd];
-    float xh[kTileRows][kNF];
+    float xh[kTileRows][kNF + 1];
     float dy[kTileRows][kNO];
     float err2[kTileRows];
 };
 
 __global__ void __launch_bounds__(kGradThreads)
     mlp_grad_kernel(const uint16_t* __restrict__ p16, const float* __restrict__ x, const float* __restrict__ t,
-                    const int* __restrict__ head, int n, float* __restrict__ partial, float* __restrict__ partial_loss) {
+                    const int* __restrict__ head, int n, int ntile, float* __restrict__ partial,
+                    float* __restrict__ partial_loss) {
     extern __shared__ float4 smem_raw[];
     GradSmem& S = *reinterpret_cast<GradSmem*>(smem_raw);
-    stage_params(p16, S.sp);
     const int tid = threadIdx.x;
-    const long r0 = (long)blockIdx.x * kTileRows;
-    if (tid < kTileRows) {
-        const long r = r0 + tid;
-        float xr[kNF], xh[kNF], y[kNO];
-        float* h1 = S.h1[tid];
-        float* h2 = S.h2[tid];
+    for (int e = tid; e < BAMG_MLP_NPARAMS; e += kGradThreads) {
+        const float v = __half2float(__ushort_as_half(p16[e]));
+        if (e < kOB1) S.w1[e / kNF][e % kNF] = v;
+        else if (e < kOW2) S.b1[e - kOB1] = v;
+        else if (e < kOB2) S.w2[(e - kOW2) / kNH][(e - kOW2) % kNH] = v;
+        else if (e < kOW3) S.b2[e - kOB2] = v;
+        else if (e < kOB3) S.w3[(e - kOW3) / kNH][(e - kOW3) % kNH] = v;
+        else if (e < kOXM) S.b3[e - kOB3] = v;
+        else if (e < kOXS) S.xm[e - kOXM] = v;
+        else S.xs[e - kOXS] = v;
+    }
+    const int row = tid / 8, g = tid & 7;        // phase 1: row of the tile, first unit
+    const int tj = tid >> 4, tk = tid & 15;      // phase 2: W2 entries (tj + 16 a, tk + 16 b)
+    float gw2[4][4] = {}, gw1[2] = {0.f, 0.f}, gsm = 0.f, loss = 0.f;
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+        __syncthreads();  // the parameters; the previous tile's phase 2
+        const long r = (long)tile * kTileRows + row;
         const bool act = r < n;
+        S.xh[row][g] = ((act ? x[r * kNF + g] : 0.f) - S.xm[g]) * S.xs[g];
+        __syncwarp();  // a row's eight threads are lanes of one warp
+        float h1[kUnits], h2[kUnits];
 #pragma unroll
-        for (int m = 0; m < kNF; ++m) xr[m] = act ? x[r * kNF + m] : 0.f;
-        row_forward(S.sp, xr, xh, h1, h2, y);
+        for (int u = 0; u < kUnits; ++u) {
+            const int k = g + 8 * u;
+            float a = 0.f;
+#pragma unroll
+            for (int m = 0; m < kNF; ++m) a = fmaf(S.w1[k][m], S.xh[row][m], a);
+            h1[u] = tanhf(a + S.b1[k]);
+            S.h1[row][k] = h1[u];
+        }
+        __syncwarp();
+        float a2[kUnits] = {};
+#pragma unroll 4
+        for (int k = 0; k < kNH; ++k) {
+            const float h = S.h1[row][k];
+#pragma unroll
+            for (int u = 0; u < kUnits; ++u) a2[u] = fmaf(S.w2[g + 8 * u][k], h, a2[u]);
+        }
+        float y0 = 0.f, y1 = 0.f;
+#pragma unroll
+        for (int u = 0; u < kUnits; ++u) {
+            const int j = g + 8 * u;
+            h2[u] = tanhf(a2[u] + S.b2[j]);
+            S.h2[row][j] = h2[u];
+            y0 = fmaf(S.w3[0][j], h2[u], y0);
+            y1 = fmaf(S.w3[1][j], h2[u], y1);
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            y0 += __shfl_xor_sync(0xffffffffu, y0, o);
+            y1 += __shfl_xor_sync(0xffffffffu, y1, o);
+        }
         float dy0 = 0.f, dy1 = 0.f, e2 = 0.f;
         if (act) {
             const int hd = head[r];
-            const float e = (hd == 0 ? y[0] : y[1]) - t[r];
+            const float e = (hd == 0 ? y0 + S.b3[0] : y1 + S.b3[1]) - t[r];
             e2 = e * e;
-            const float g = 2.f * e / (float)n;
-            dy0 = hd == 0 ? g : 0.f;
-            dy1 = hd == 0 ? 0.f : g;
+            const float gr = 2.f * e / (float)n;
+            dy0 = hd == 0 ? gr : 0.f;
+            dy1 = hd == 0 ? 0.f : gr;
         }
-        S.dy[tid][0] = dy0;
-        S.dy[tid][1] = dy1;
-        S.err2[tid] = e2;
+        if (g == 0) {
+            S.dy[row][0] = dy0;
+            S.dy[row][1] = dy1;
+            S.err2[row] = e2;
+        }
 #pragma unroll
-        for (int m = 0; m < kNF; ++m) S.xh[tid][m] = xh[m];
-        float* da2 = S.da2[tid];
+        for (int u = 0; u < kUnits; ++u) {
+            const int j = g + 8 * u;
+            S.da2[row][j] = (dy0 * S.w3[0][j] + dy1 * S.w3[1][j]) * (1.f - h2[u] * h2[u]);
+        }
+        __syncwarp();
+        float a1[kUnits] = {};
+#pragma unroll 4
         for (int j = 0; j < kNH; ++j) {
-            const float g = dy0 * S.sp[kOW3 + j] + dy1 * S.sp[kOW3 + kNH + j];
-            da2[j] = g * (1.f - h2[j] * h2[j]);
+            const float d = S.da2[row][j];
+#pragma unroll
+            for (int u = 0; u < kUnits; ++u) a1[u] = fmaf(S.w2[j][g + 8 * u], d, a1[u]);
         }
-        for (int k = 0; k < kNH; ++k) {
-            float g = 0.f;
+#pragma unroll
+        for (int u = 0; u < kUnits; ++u) S.da1[row][g + 8 * u] = a1[u] * (1.f - h1[u] * h1[u]);
+        __syncthreads();
+#pragma unroll 2
+        for (int q = 0; q < kTileRows; ++q) {
+            float dj[4], hk[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                dj[u] = S.da2[q][tj + 16 * u];
+                hk[u] = S.h1[q][tk + 16 * u];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) gw2[u][v] = fmaf(dj[u], hk[v], gw2[u][v]);
+        }
+        // W1: entries tid and tid + 256 of 512; then b1, b2, W3 (one each) and b3, loss
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int k = (tid + u * kGradThreads) / kNF, m = (tid + u * kGradThreads) % kNF;
 #pragma unroll 8
-            for (int j = 0; j < kNH; ++j) g = fmaf(S.sp[kOW2 + j * kNH + k], da2[j], g);
-            S.da1[tid][k] = g * (1.f - h1[k] * h1[k]);
+            for (int q = 0; q < kTileRows; ++q) gw1[u] = fmaf(S.da1[q][k], S.xh[q][m], gw1[u]);
         }
-    }
-    __syncthreads();
-    float* out = partial + (size_t)blockIdx.x * BAMG_MLP_NTRAIN;
-    // W2 and b2 (4096 + 64 outputs), W1 and b1 (512 + 64), W3 and b3 (128 + 2)
-    for (int o = tid; o < BAMG_MLP_NTRAIN; o += kGradThreads) {
-        float acc = 0.f;
-        if (o >= kOW2 && o < kOB2) {
-            const int j = (o - kOW2) / kNH, k = (o - kOW2) % kNH;
-            for (int r = 0; r < kTileRows; ++r) acc = fmaf(S.da2[r][j], S.h1[r][k], acc);
-        } else if (o >= kOB2 && o < kOW3) {
-            const int j = o - kOB2;
-            for (int r = 0; r < kTileRows; ++r) acc += S.da2[r][j];
-        } else if (o < kOB1) {
-            const int k = o / kNF, m = o % kNF;
-            for (int r = 0; r < kTileRows; ++r) acc = fmaf(S.da1[r][k], S.xh[r][m], acc);
-        } else if (o < kOW2) {
-            const int k = o - kOB1;
-            for (int r = 0; r < kTileRows; ++r) acc += S.da1[r][k];
-        } else if (o < kOB3) {
-            const int q = o - kOW3, oo = q / kNH, j = q % kNH;
-            for (int r = 0; r < kTileRows; ++r) acc = fmaf(S.dy[r][oo], S.h2[r][j], acc);
+        if (tid < kNH) {
+#pragma unroll 8
+            for (int q = 0; q < kTileRows; ++q) gsm += S.da1[q][tid];
+        } else if (tid < 2 * kNH) {
+#pragma unroll 8
+            for (int q = 0; q < kTileRows; ++q) gsm += S.da2[q][tid - kNH];
         } else {
-            const int oo = o - kOB3;
-            for (int r = 0; r < kTileRows; ++r) acc += S.dy[r][oo];
+            const int o = (tid - 2 * kNH) / kNH, j = (tid - 2 * kNH) % kNH;
+#pragma unroll 8
+            for (int q = 0; q < kTileRows; ++q) gsm = fmaf(S.dy[q][o], S.h2[q][j], gsm);
         }
-        out[o] = acc;
+        if (tid < kNO) {  // (b3: a second small sum of these threads, kept with the loss)
+            for (int q = 0; q < kTileRows; ++q) loss += S.dy[q][tid];
+        } else if (tid == kNO) {
+            for (int q = 0; q < kTileRows; ++q) loss += S.err2[q];
+        }
     }
-    if (tid == 0) {
-        float l = 0.f;
-        for (int r = 0; r < kTileRows; ++r) l += S.err2[r];
-        partial_loss[blockIdx.x] = l;
-    }
+    float* out = partial + (size_t)blockIdx.x * BAMG_MLP_NTRAIN;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) out[kOW2 + (tj + 16 * u) * kNH + tk + 16 * v] = gw2[u][v];
+    out[kOW1 + tid] = gw1[0];
+    out[kOW1 + tid + kGradThreads] = gw1[1];
+    if (tid < kNH) out[kOB1 + tid] = gsm;
+    else if (tid < 2 * kNH) out[kOB2 + tid - kNH] = gsm;
+    else out[kOW3 + tid - 2 * kNH] = gsm;
+    if (tid < kNO) out[kOB3 + tid] = loss;
+    else if (tid == kNO) partial_loss[blockIdx.x] = loss;
 }
+static_assert(kNH * kNF == 2 * kGradThreads && kGradThreads == 4 * kNH && kNO == 2 && kTileRows * 8 == kGradThreads,
+              "work split of mlp_grad_kernel");
 
-// grad[o] = sum over tiles (ascending) of partial[tile][o]; loss likewise / n
-__global__ void grad_reduce_kernel(int ntile, int n, const float* __restrict__ partial,
-                                   const float* __restrict__ partial_loss, float* __restrict__ grad,
-                                   float* __restrict__ loss) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
+// grad[o] = sum over the CTAs of partial[CTA][o]: a CTA takes 32 outputs, warp w
+// the w-th eighth of the CTAs in ascending order, then the eighths in order;
+// output NTRAIN is the loss, divided by n
+__global__ void __launch_bounds__(256) grad_reduce_kernel(int nctas, int n, const float* __restrict__ partial,
+                                                          const float* __restrict__ partial_loss,
+                                                          float* __restrict__ grad, float* __restrict__ loss) {
+    __shared__ float sh[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int o = blockIdx.x * 32 + lane;
+    const int per = (nctas + 7) / 8, c0 = w * per, c1 = min(nctas, c0 + per);
+    float s = 0.f;
     if (o < BAMG_MLP_NTRAIN) {
-        float s = 0.f;
-        for (int tt = 0; tt < ntile; ++tt) s += partial[(size_t)tt * BAMG_MLP_NTRAIN + o];
-        grad[o] = s;
+#pragma unroll 8
+        for (int c = c0; c < c1; ++c) s += partial[(size_t)c * BAMG_MLP_NTRAIN + o];
+    } else if (o == BAMG_MLP_NTRAIN) {
+        for (int c = c0; c < c1; ++c) s += partial_loss[c];
     }
-    if (o == 0) {
-        float s = 0.f;
-        for (int tt = 0; tt < ntile; ++tt) s += partial_loss[tt];
-        *loss = s / (float)n;
-    }
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w != 0 || o > BAMG_MLP_NTRAIN) return;
+    s = 0.f;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) s += sh[v][lane];
+    if (o < BAMG_MLP_NTRAIN) grad[o] = s;
+    else *loss = s / (float)n;
 }
 
-size_t mlp_grad_workspace(int n) {
+static int grad_ctas(int n) {
     const int ntile = ceil_div(n, kTileRows);
-    return sizeof(float) * ((size_t)ntile * BAMG_MLP_NTRAIN + (size_t)ntile);
+    return ntile < kGradCtas ? ntile : kGradCtas;
+}
+size_t mlp_grad_workspace(int n) {
+    return sizeof(float) * (size_t)grad_ctas(n) * (BAMG_MLP_NTRAIN + 1);
 }
 
 int launch_mlp_grad(const uint16_t* p16, const float* x, const float* t, const int* head, int n, float* grad,
                     float* loss, float* work, cudaStream_t s) {
     if (n < 1) return BAMG_EINVAL;
-    const int ntile = ceil_div(n, kTileRows);
+    const int nctas = grad_ctas(n);
     const size_t smem = sizeof(GradSmem);
     // more than 48 KB of dynamic shared memory needs the opt-in (idempotent)
     BAMG_CUDA_TRY(cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     float* partial = work;
-    float* partial_loss = work + (size_t)ntile * BAMG_MLP_NTRAIN;
-    mlp_grad_kernel<<<ntile, kGradThreads, smem, s>>>(p16, x, t, head, n, partial, partial_loss);
-    grad_reduce_kernel<<<ceil_div(BAMG_MLP_NTRAIN, 256), 256, 0, s>>>(ntile, n, partial, partial_loss, grad, loss);
+    float* partial_loss = work + (size_t)nctas * BAMG_MLP_NTRAIN;
+    mlp_grad_kernel<<<nctas, kGradThreads, smem, s>>>(p16, x, t, head, n, ceil_div(n, kTileRows), partial,
+                                                      partial_loss);
+    grad_reduce_kernel<<<ceil_div(BAMG_MLP_NTRAIN + 1, 32), 256, 0, s>>>(nctas, n, partial, partial_loss, grad, loss);
     return launched(2);
 }
 
