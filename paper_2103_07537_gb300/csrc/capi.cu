@@ -3053,8 +3053,17 @@ extern "C" int bsr_spmv(const int* row_ptr, const int* col_idx, const double* va
                         const double* x, double* y, void* stream) {
     if (!row_ptr || !col_idx || !vals || !x || !y || n_nodes < 0 || b < 1 || b > kMaxB || x == y)
         return BAMG_EINVAL;
-    return launch_spmv<double>(b, b, 0, n_nodes, row_ptr, col_idx, vals, x, nullptr, y,
-                               static_cast<cudaStream_t>(stream));
+    // By scalar rows (the row lengths are on the device): a warp per block row
+    // for small matrices (shortest chains), four lanes per scalar row where
+    // those leave the FP64 pipe half used by reductions, a thread per scalar row
+    // once that alone fills the GPU.  us per product, warp / split / thread:
+    // 3D b = 4: 37044 rows 14.5 / 12.5 / 14.5, 97556 rows 31.0 / 26.1 / 24.8,
+    // 1098500 rows 330 / 240 / 208; 2D b = 1: 9409 rows 8.3 / 4.5 / 4.4; 2D b = 6:
+    // 25350 rows 8.3 / 8.3 / 8.5, 99846 rows 19.4 / 18.7 / 14.6.
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const long rows = (long)n_nodes * b;
+    if (rows < 8192) return launch_spmv<double>(b, b, 0, n_nodes, row_ptr, col_idx, vals, x, nullptr, y, s);
+    return launch_spmv_tpr<double>(b, b, 0, n_nodes, row_ptr, col_idx, vals, x, nullptr, y, s, rows < 65536 ? 1 : 0);
 }
 
 // ---------------------------------------------------------------------------
