@@ -2526,7 +2526,16 @@ static int ensure_graph(bamg_ctx* h) {
     BAMG_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     long long kernels = 0;
     t_capture_sink = &kernels;
-    int st = cycle_direct(h, h->cyc_in, h->cyc_out, cs);
+    int st;
+    if (h->p.cycle_prec == 64) {
+        st = cycle_direct(h, h->cyc_in, h->cyc_out, cs);
+    } else {
+        // the casts at the FP32 cycle's boundary read and write the caller's
+        // vectors and stay outside the graph: no staging copies
+        PdlScope pdl(h->p.use_pdl != 0);
+        st = mgv<float>(h, 0, h->r32, h->z32, cs);
+        h->prof_level = -1;
+    }
     t_capture_sink = nullptr;
     h->graph_kernels = kernels;
     cudaGraph_t g = nullptr;
@@ -2590,7 +2599,14 @@ static int apply_impl(bamg_ctx* h, const double* r, double* z, cudaStream_t s) {
     // (a cycle with the cooperative grid tail is one launch plus casts: direct)
     if (!h->p.use_graph || h->prof || h->tail_grid) return cycle_direct(h, r, z, s);
     TRY(ensure_graph(h));
-    const size_t nbytes = sizeof(double) * (size_t)h->lev[0].n * h->b;
+    const long N = (long)h->lev[0].n * h->b;
+    if (h->p.cycle_prec == 32) {
+        TRY(launch_cast_d2f(N, r, h->r32, s));
+        BAMG_CUDA_TRY(cudaGraphLaunch(h->graph_exec, s));
+        note_launch((int)h->graph_kernels);
+        return launch_cast_f2d(N, h->z32, z, s);
+    }
+    const size_t nbytes = sizeof(double) * (size_t)N;
     BAMG_CUDA_TRY(cudaMemcpyAsync(h->cyc_in, r, nbytes, cudaMemcpyDeviceToDevice, s));
     BAMG_CUDA_TRY(cudaGraphLaunch(h->graph_exec, s));
     note_launch((int)h->graph_kernels);

@@ -1179,31 +1179,40 @@ template int tail_cluster_size<float>(int, int, int);
 // ---------------------------------------------------------------------------
 // precision casts at the cycle boundary (FP64 Krylov vectors <-> FP32 cycle)
 // ---------------------------------------------------------------------------
-__global__ void cast_d2f_kernel(long m, const double* __restrict__ x, float* __restrict__ y) {
+// Y[e] = X[e], two at a time (V2 = 1) where both vectors allow it: the FP64 side
+// in 16-byte loads or stores
+template <typename X, typename Y, bool V2>
+__global__ void cast_kernel(long m, const X* __restrict__ x, Y* __restrict__ y) {
     pdl_wait();
     pdl_trigger();
-    for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (long)gridDim.x * blockDim.x)
-        y[e] = (float)x[e];
+    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long)gridDim.x * blockDim.x;
+    if constexpr (V2) {
+        using X2 = typename VecOf<X>::v2;
+        using Y2 = typename VecOf<Y>::v2;
+        for (long e = t; e < m / 2; e += nt) {
+            const X2 v = reinterpret_cast<const X2*>(x)[e];
+            Y2 w;
+            w.x = (Y)v.x;
+            w.y = (Y)v.y;
+            reinterpret_cast<Y2*>(y)[e] = w;
+        }
+        if (t == 0 && (m & 1)) y[m - 1] = (Y)x[m - 1];
+    } else {
+        for (long e = t; e < m; e += nt) y[e] = (Y)x[e];
+    }
 }
-__global__ void cast_f2d_kernel(long m, const float* __restrict__ x, double* __restrict__ y) {
-    pdl_wait();
-    pdl_trigger();
-    for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (long)gridDim.x * blockDim.x)
-        y[e] = (double)x[e];
-}
-static int grid_for(long m) {
-    long g = (m + 255) / 256;
-    return (int)(g < 152L * 16 ? (g > 0 ? g : 1) : 152L * 16);
-}
-int launch_cast_d2f(long m, const double* x, float* y, cudaStream_t s) {
+template <typename X, typename Y>
+static int launch_cast(long m, const X* x, Y* y, cudaStream_t s) {
     if (m <= 0) return BAMG_OK;
-    if (launch_k(cast_d2f_kernel, grid_for(m), 256, 0, s, m, x, y) != cudaSuccess) return BAMG_ECUDA;
-    return launched(1);
+    const bool v2 = (reinterpret_cast<uintptr_t>(x) % (2 * sizeof(X))) == 0 &&
+                    (reinterpret_cast<uintptr_t>(y) % (2 * sizeof(Y))) == 0;
+    const long items = v2 ? (m + 1) / 2 : m, g = (items + 255) / 256;
+    const int grid = (int)(g < 152L * 16 ? g : 152L * 16);
+    const cudaError_t e = v2 ? launch_k(cast_kernel<X, Y, true>, grid, 256, 0, s, m, x, y)
+                             : launch_k(cast_kernel<X, Y, false>, grid, 256, 0, s, m, x, y);
+    return e == cudaSuccess ? launched(1) : BAMG_ECUDA;
 }
-int launch_cast_f2d(long m, const float* x, double* y, cudaStream_t s) {
-    if (m <= 0) return BAMG_OK;
-    if (launch_k(cast_f2d_kernel, grid_for(m), 256, 0, s, m, x, y) != cudaSuccess) return BAMG_ECUDA;
-    return launched(1);
-}
+int launch_cast_d2f(long m, const double* x, float* y, cudaStream_t s) { return launch_cast(m, x, y, s); }
+int launch_cast_f2d(long m, const float* x, double* y, cudaStream_t s) { return launch_cast(m, x, y, s); }
 
 }  // namespace bamg
