@@ -292,6 +292,10 @@ struct bamg_ctx {
     double tail_bytes = 0.0, tail_flops = 0.0;
     std::vector<TailPhase>* rec = nullptr;  // set while the tail phases are recorded
     double rec_bytes = 0.0, rec_flops = 0.0;
+    // the levels from l_cc down in one cluster launch per cycle (k_coarse.cu)
+    int l_cc = -1;
+    CcArgs cc{};
+    double cc_bytes = 0.0, cc_flops = 0.0;
     // profiling
     int prof = 0;
     std::vector<ProfRec> recs;        // direct launches, resolved when read
@@ -551,6 +555,7 @@ extern "C" const char* amg_strerror(int status) {
 // setup
 // ---------------------------------------------------------------------------
 static int setup_tail(bamg_ctx* h, cudaStream_t s);
+static int setup_coarse_cycle(bamg_ctx* h, cudaStream_t s);
 static int record_tail(bamg_ctx* h, cudaStream_t s, bool only_counts);
 
 using Clock = std::chrono::steady_clock;
@@ -1730,6 +1735,7 @@ static int setup_impl(bamg_ctx* h, const int* row_ptr, const int* col_idx, const
         else TRY(autotune_levels<float>(h, s));
     }
     if (h->nsys == 1 && h->nf == 1) TRY(setup_tail(h, s));
+    TRY(setup_coarse_cycle(h, s));
     h->t_phase[6] += ms_since(tp);
     return BAMG_OK;
 }
@@ -2267,6 +2273,10 @@ static int mgv(bamg_ctx* h, int l, const T* rhs, T* out, cudaStream_t s) {
                launch_tail<T>(b, h->fb, h->tail_d, h->n_tail, h->tail_cluster, s));
         return BAMG_OK;
     }
+    if (!h->rec && l == h->l_cc) {  // this level and all below in one cluster launch
+        PL(BAMG_K_TAIL, h->cc_bytes, h->cc_flops, launch_coarse_cycle<T>(b, h->fb, h->cc, rhs, out, s));
+        return BAMG_OK;
+    }
     if (l == h->nlev - 1 && h->nsys > 1) {  // one dense inverse per system
         const Level& Lc = h->lev[l];
         PL(BAMG_K_COARSE, 0.0, 0.0,
@@ -2518,6 +2528,124 @@ static int setup_tail(bamg_ctx* h, cudaStream_t s) {
     }
     h->l_tail = lt;
     return record_tail(h, s, false);
+}
+
+// The coarse levels whose rows and vectors fit the shared memory of one cluster
+// run as one launch per cycle, from the finest such level down, in the default
+// configuration (the forced row mappings, the recorded tail and the other
+// sub-solvers keep their own launches).  Wherever they fit they are the faster
+// form: a colour step of up to 1200 nodes takes 0.9 to 1.6 us inside the cluster
+// and 2.1 to 2.5 us as a kernel.
+static int setup_coarse_cycle(bamg_ctx* h, cudaStream_t s) {
+    h->l_cc = -1;
+    const amg_params& p = h->p;
+    if (h->nsys != 1 || h->nf != 1 || h->nlev < 2 || h->tail_d || p.sub_solver != 0 || p.inner_sweeps > 1 ||
+        p.autotune != 1 || p.sweep != 0 || p.tail_dofs != 0)
+        return BAMG_OK;
+    const int b = h->b, fb = h->fb, F = h->F, last = h->nlev - 1;
+    const bool f64 = p.cycle_prec == 64;
+    const size_t es = f64 ? sizeof(double) : sizeof(float);
+    const int ctas = kCcCtas;
+    constexpr int kMaxNodes = 16 * 1024;  // (no level beyond this fits)
+    auto per_of = [&](int l) { return ceil_div(h->lev[l].n, ctas); };
+    int lo = last;
+    while (lo > 0 && last - lo + 1 < kCcLevels && !h->lev[lo - 1].smoothed && !h->lev[lo - 1].fm &&
+           h->lev[lo - 1].n <= kMaxNodes && h->lev[lo - 1].sweep == 0)
+        --lo;
+    if (lo == last) return BAMG_OK;
+    // stored blocks at the CTAs' first nodes, every candidate level
+    const int nc = last - lo, bs = ctas + 1;
+    int* bound = nullptr;
+    TRY(h->alloc(&bound, (size_t)nc * bs));
+    for (int l = lo; l < last; ++l)
+        TRY(launch_cc_bound(h->lev[l].n, per_of(l), ctas, h->lev[l].rp, bound + (l - lo) * bs, s));
+    std::vector<int> hb((size_t)nc * bs);
+    BAMG_CUDA_TRY(cudaMemcpyAsync(hb.data(), bound, sizeof(int) * hb.size(), cudaMemcpyDeviceToHost, s));
+    BAMG_CUDA_TRY(cudaStreamSynchronize(s));
+    h->release(bound);
+    // the slices, from the coarsest level up while they fit
+    CcLevel lv[kCcLevels] = {};
+    size_t smem = 0;
+    int first = last;
+    for (int l = last; l >= lo; --l) {
+        CcLevel& C = lv[l - lo];
+        const Level& L = h->lev[l];
+        C.n = L.n;
+        C.per = per_of(l);
+        C.colours = L.n_colours;
+        const size_t per = (size_t)C.per;
+        size_t at = smem;
+        auto slot = [&](int which, size_t bytes, bool copied) {
+            C.off[which] = (int)at;
+            at += (bytes + (copied ? 32 : 0) + 15) / 16 * 16;
+        };
+        slot(kCcX0, per * b * es, false);
+        slot(kCcX1, l < last ? per * b * es : 0, false);
+        slot(kCcRhs, per * b * es, false);
+        slot(kCcXt, l < last ? per * fb * es : (size_t)h->nd * es, false);
+        if (l < last) {
+            size_t nk = 0;
+            const int* q = hb.data() + (size_t)(l - lo) * bs;
+            for (int r = 0; r < ctas; ++r) nk = std::max(nk, (size_t)(q[r + 1] - q[r]));
+            slot(kCcRp, (per + 1) * sizeof(int), true);
+            slot(kCcVals, nk * b * b * es, true);
+            slot(kCcEnc, nk * sizeof(int), true);
+            slot(kCcLow, nk, true);
+            slot(kCcDinv, per * F * fb * fb * es, true);
+            slot(kCcOmega, (f64 ? (void*)L.omega_s64 : (void*)L.omega_s32) ? per * F * es : 0, true);
+            slot(kCcList, per * sizeof(int), true);
+            slot(kCcListOff, ((size_t)C.colours + 1) * sizeof(int), true);
+            slot(kCcAgg, per * sizeof(int), true);
+        }
+        if (at > (size_t)kCcMaxSmem) break;
+        smem = at;
+        first = l;
+    }
+    if (first >= last || !coarse_cycle_fits(b, fb, f64, ctas, smem)) return BAMG_OK;
+    double bytes = 0.0, flops = 0.0;
+    for (int l = first; l < last; ++l) {
+        CcLevel& C = lv[l - lo];
+        const Level& L = h->lev[l];
+        int *enc = nullptr, *list = nullptr, *off = nullptr, *agg = nullptr, *mem = nullptr;
+        TRY(h->alloc(&enc, (size_t)L.nnzb));
+        TRY(h->alloc(&list, (size_t)L.n));
+        TRY(h->alloc(&off, (size_t)ctas * (L.n_colours + 1)));
+        TRY(h->alloc(&agg, (size_t)L.n));
+        TRY(h->alloc(&mem, (size_t)L.n));
+        TRY(launch_cc_encode(L.nnzb, C.per, L.ci, enc, s));
+        TRY(launch_cc_list(L.n, C.per, ctas, L.n_colours, L.colour, list, off, s));
+        TRY(launch_cc_encode(L.n, lv[l + 1 - lo].per, L.agg, agg, s));
+        TRY(launch_cc_encode(L.n, C.per, L.members, mem, s));
+        C.rp = L.rp;
+        C.vals = f64 ? (const void*)L.vals64 : (const void*)L.vals32;
+        C.enc = enc;
+        C.lowk = L.lowk;
+        C.dinv = f64 ? (const void*)L.dinv64 : (const void*)L.dinv32;
+        C.omega = f64 ? (const void*)L.omega_s64 : (const void*)L.omega_s32;
+        C.list = list;
+        C.list_off = off;
+        C.agg = agg;
+        C.agg_ptr = L.agg_ptr;
+        C.members = mem;
+        for (int r = 0; r <= ctas; ++r) C.bound[r] = hb[(size_t)(l - lo) * bs + r];
+        bytes += (double)L.nnzb * (b * b * es + 5.0) + (double)L.n * (F * fb * fb * es + 20.0);
+        flops += 2.0 * L.nnzb * b * b * (p.n_pre + p.n_post + 1);
+    }
+    bytes += (double)h->nd * h->nd * (h->coarse_inv32 ? 4.0 : 8.0) + 2.0 * h->lev[first].n * b * es;
+    h->cc = CcArgs{};
+    h->cc.nlev = last - first + 1;
+    for (int l = first; l <= last; ++l) h->cc.lev[l - first] = lv[l - lo];
+    h->cc.ctas = ctas;
+    h->cc.n_pre = p.n_pre;
+    h->cc.n_post = p.n_post;
+    h->cc.smem = (int)smem;
+    h->cc.omega = p.omega;
+    h->cc.inv64 = h->coarse_inv32 ? nullptr : h->coarse_inv;
+    h->cc.inv32 = h->coarse_inv32;
+    h->cc_bytes = bytes;
+    h->cc_flops = flops + 2.0 * h->nd * h->nd;
+    h->l_cc = first;
+    return BAMG_OK;
 }
 
 static int ensure_graph(bamg_ctx* h) {
@@ -3142,7 +3270,7 @@ extern "C" int amg_stats(bamg_t h, char* json, int cap) {
         snprintf(buf, sizeof buf, "%s\"%s\":%.4f", q ? "," : "", names[q], h->t_phase[q]);
         o += buf;
     }
-    o += "},\"tail_level\":" + std::to_string(h->l_tail) + ",\"tail_phases\":" + std::to_string(h->n_tail) +
+    o += "},\"coarse_cycle_level\":" + std::to_string(h->l_cc) + ",\"tail_level\":" + std::to_string(h->l_tail) + ",\"tail_phases\":" + std::to_string(h->n_tail) +
          ",\"tail_cluster\":" + std::to_string(h->tail_cluster) + ",\"tail_grid\":" + std::to_string(h->tail_grid) +
          ",\"levels\":[";
     for (int l = 0; l < h->nlev; ++l) {
@@ -3396,6 +3524,7 @@ extern "C" int amg_set_omega(bamg_t h, int level, const double* omega_s, void* s
         BAMG_CUDA_TRY(cudaStreamSynchronize(h->stream));
         drop_graphs(h);
         if (h->tail_d) TRY(record_tail(h, h->stream, false));
+        if (h->l_cc >= 0) TRY(setup_coarse_cycle(h, h->stream));
     }
     BAMG_CUDA_TRY(cudaMemcpyAsync(L.omega_s64, omega_s, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
     if (h->p.cycle_prec == 32) TRY(launch_convert_d2f((long)m, L.omega_s64, L.omega_s32, s));

@@ -497,6 +497,44 @@ int grid_tail_size(int b, int fb);
 // largest resident cluster size <= want for the tail kernel (0: none)
 template <typename T>
 int tail_cluster_size(int b, int fb, int want);
+// ---- the coarse levels of a cycle in one cluster launch (k_coarse.cu) ----
+constexpr int kCcLevels = 8;
+constexpr int kCcCtas = 16;
+constexpr int kCcMaxSmem = 216 * 1024;  // dynamic shared memory of a CTA
+// places of a level's slices in the shared memory of a CTA
+enum CcSlot : int { kCcX0, kCcX1, kCcRhs, kCcXt, kCcRp, kCcVals, kCcEnc, kCcLow, kCcDinv, kCcOmega, kCcList,
+                    kCcListOff, kCcAgg, kCcSlots };
+struct CcLevel {
+    int n, per, colours;   // CTA c owns nodes c * per .. (c + 1) * per - 1
+    int off[kCcSlots];     // byte offsets, multiples of 16
+    const int* rp;
+    const void* vals;
+    const int* enc;        // columns as (owner << 16 | local)
+    const unsigned char* lowk;
+    const void* dinv;
+    const void* omega;     // damping of every node and field, or null
+    const int* list;       // own nodes by colour, local
+    const int* list_off;
+    const int* agg;        // aggregates as (owner << 16 | local) of the next level
+    const int* agg_ptr;
+    const int* members;    // members as (owner << 16 | local) of this level
+    int bound[kCcCtas + 1];  // rp at the CTAs' first nodes
+};
+struct CcArgs {
+    int nlev = 0, ctas = 0, n_pre = 0, n_post = 0, smem = 0;
+    double omega = 0.0;
+    CcLevel lev[kCcLevels] = {};    // (in the kernel's parameters: no loads ahead of the copies)
+    const double* inv64 = nullptr;  // the coarsest inverse, FP64 or FP32
+    const float* inv32 = nullptr;
+};
+template <typename T>
+int launch_coarse_cycle(int b, int fb, const CcArgs& a, const T* rhs, T* out, cudaStream_t s);
+bool coarse_cycle_fits(int b, int fb, bool fp64, int ctas, size_t smem);
+int launch_cc_encode(long m, int per, const int* idx, int* enc, cudaStream_t s);
+int launch_cc_list(int n, int per, int ctas, int colours, const int* colour, int* list, int* list_off,
+                   cudaStream_t s);
+int launch_cc_bound(int n, int per, int ctas, const int* ptr, int* bound, cudaStream_t s);
+
 // y = Ainv x for the dense nd x nd inverse of type S (double or float; the
 // sum in S), x, y of type T
 template <typename T, typename S>
