@@ -1043,30 +1043,41 @@ static int autotune_levels(bamg_ctx* h, cudaStream_t s) {
         }
         if (L.bgs_tpr == 4 && L.tune_us[6] >= 1e29f) L.bgs_tpr = 3;  // the staged kernel does not take this level
         if ((L.bgs_tpr == 6 || L.bgs_tpr == 7) && !bsp_supported(b, h->fb)) L.bgs_tpr = 3;  // block too large
-        if (h->p.autotune == 1 && h->p.use_pdl && (L.bgs_tpr == 0 || L.bgs_tpr == 5)) {
-            // warp against four warps per node again, as a whole field step
-            // (every colour of field 0) in the cycle's launch mode: with
-            // programmatic dependent launches each kernel's loads before its
-            // wait overlap the previous colour, which favours the wider mapping
-            // (3D level 1: 7% faster in the cycle, within 3% one colour alone)
+        if (h->p.autotune == 1 && h->p.use_pdl && !big) {
+            // the leading mappings again, as the cycle runs them: a step from
+            // zero and a step from an iterate, every colour of field 0, in
+            // programmatic dependent launches (each kernel's loads before its
+            // wait overlap the previous colour, which one colour launched
+            // alone does not show: 3D level 1, four warps per node 7% faster in
+            // the cycle and within 3% alone; 2D 128^2 level 0 FP64, four lanes
+            // per row against warp per node: cycle 207 against 221 us, alone a
+            // near tie that went either way)
             PdlScope pdl(true);
             const int c_hi = h->nf > 1 ? L.fcol[1] : L.n_colours;
-            float tstep[2] = {0.f, 0.f};
-            for (int m = 0; m < 2; ++m) {
-                L.bgs_tpr = m == 0 ? 0 : 5;
-                tstep[m] = time_launch(s, e0, e1, reps, [&]() {
-                    for (int c = 0; c < c_hi; ++c) {
-                        BgsArgs ac = a;
-                        ac.n_in_colour = L.colour_ptr[c + 1] - L.colour_ptr[c];
-                        ac.nodes = L.colour_nodes + L.colour_ptr[c];
-                        ac.colour = c;
-                        const int st = launch_colour_step<T>(h, L, ac, s);
-                        if (st != BAMG_OK) return st;
-                    }
+            const int lead = L.bgs_tpr;
+            int best_m = 0;
+            float best_us = 1e30f;
+            for (int m : {0, 5, 3, lead}) {
+                L.bgs_tpr = m;
+                const float us = time_launch(s, e0, e1, reps, [&]() {
+                    for (int t = 0; t < 2; ++t)
+                        for (int c = 0; c < c_hi; ++c) {
+                            BgsArgs ac = a;
+                            if (t == 0) ac.x_in = nullptr;
+                            ac.n_in_colour = L.colour_ptr[c + 1] - L.colour_ptr[c];
+                            ac.nodes = L.colour_nodes + L.colour_ptr[c];
+                            ac.colour = c;
+                            const int st = launch_colour_step<T>(h, L, ac, s);
+                            if (st != BAMG_OK) return st;
+                        }
                     return (int)BAMG_OK;
                 });
+                if (us < best_us) {
+                    best_us = us;
+                    best_m = m;
+                }
             }
-            L.bgs_tpr = tstep[1] < tstep[0] ? 5 : 0;
+            L.bgs_tpr = best_m;
         }
         L.spmv_tpr = h->p.autotune >= 2 || (h->p.autotune == 1 && L.tune_us[3] < kTuneMargin * L.tune_us[2]);
         // one whole field step (every colour of field 0) as per-colour launches

@@ -108,63 +108,79 @@ __device__ __forceinline__ bool last_cta(unsigned* ticket) {
     return last;
 }
 
-// out[v] = sum of the chunk partials partial[v * nchunk + c], one warp per v;
-// lane l sums chunks l, l+32, ... in four interleaved accumulators (their loads
-// are independent), a fixed order for a fixed chunk count
+// out[v] = sum of the chunk partials partial[v * nchunk + c], a warp for four v
+// at a time (their loads together); lane l sums chunks l, l+32, ... in four
+// interleaved accumulators, a fixed order for a fixed chunk count
 __device__ __forceinline__ void finish_sums(int nv, const double* partial, double* out) {
-    const int lane = threadIdx.x & 31;
+    constexpr int VU = 4;
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const int nchunk = gridDim.x;
-    for (int v = threadIdx.x >> 5; v < nv; v += blockDim.x >> 5) {
-        const double* p = partial + (size_t)v * nchunk;
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        int c = lane;
-        for (; c + 96 < nchunk; c += 128) {
-            s0 += __ldcg(p + c);
-            s1 += __ldcg(p + c + 32);
-            s2 += __ldcg(p + c + 64);
-            s3 += __ldcg(p + c + 96);
+    for (int v0 = threadIdx.x >> 5; v0 < nv; v0 += nw * VU) {
+        double s[VU][4];
+#pragma unroll
+        for (int u = 0; u < VU; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[u][q] = 0.0;
+        for (int c = lane; c < nchunk; c += 128)
+#pragma unroll
+            for (int u = 0; u < VU; ++u) {
+                const int v = v0 + u * nw;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (v < nv && c + 32 * q < nchunk) s[u][q] += __ldcg(partial + (size_t)v * nchunk + c + 32 * q);
+            }
+#pragma unroll
+        for (int u = 0; u < VU; ++u) {
+            const int v = v0 + u * nw;
+            if (v >= nv) break;  // (uniform)
+            const double t = warp_sum((s[u][0] + s[u][1]) + (s[u][2] + s[u][3]));
+            if (lane == 0) out[v] = t;
         }
-        for (; c < nchunk; c += 32) s0 += __ldcg(p + c);
-        double s = (s0 + s1) + (s2 + s3);
-        s = warp_sum(s);
-        if (lane == 0) out[v] = s;
     }
 }
 
-// Arnoldi bookkeeping (one thread): column j of the Hessenberg matrix from
-// h1 + h2 and ||w||, breakdown test, previous rotations, the new rotation,
-// the residual estimate |g_{j+1}|.  scal = {h_{j+1,j}, |g_{j+1}|, breakdown,
-// ||w|| before orthogonalising}.
-__device__ void givens_update(const GivensArgs& a, double wsq) {
-    const int j = a.j, m = a.m;
+// Arnoldi bookkeeping by the whole CTA: column j of the Hessenberg matrix from
+// h1 (+ h2) and ||w||, breakdown test, previous rotations, the new rotation, the
+// residual estimate |g_{j+1}|.  scal = {h_{j+1,j}, |g_{j+1}|, breakdown, ||w||
+// before orthogonalising}.  The column and the rotations are loaded and stored
+// by all threads; one thread applies them in shared memory (a chain of two FP64
+// operations per rotation; through global memory it took 15 us at step 50).
+__device__ void givens_update(const GivensArgs& a, double wsq, bool with_h2) {
+    __shared__ double col[kMaxRestart + 2], cs[kMaxRestart], sn[kMaxRestart];
+    const int j = a.j, m = a.m, t = threadIdx.x;
     double* H = a.H;
-    const double wn0 = sqrt(__ldcg(a.h1 + j + 1));  // ||w||^2 before orthogonalising
-    for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = __ldcg(a.h1 + i) + __ldcg(a.h2 + i);
-    const double hn = sqrt(wsq);
-    H[(size_t)(j + 1) * m + j] = hn;
-    const int breakdown = !(hn > 1e-14 * wn0);
-    for (int i = 0; i < j; ++i) {
-        const double x0 = H[(size_t)i * m + j], x1 = H[(size_t)(i + 1) * m + j];
-        H[(size_t)i * m + j] = a.cs[i] * x0 + a.sn[i] * x1;
-        H[(size_t)(i + 1) * m + j] = -a.sn[i] * x0 + a.cs[i] * x1;
+    const double wn0 = sqrt(__ldcg(a.h1 + j + 1));  // ||w|| before orthogonalising
+    if (t <= j) col[t] = __ldcg(a.h1 + t) + (with_h2 ? __ldcg(a.h2 + t) : 0.0);
+    if (t < j) {
+        cs[t] = __ldcg(a.cs + t);
+        sn[t] = __ldcg(a.sn + t);
     }
-    const double x0 = H[(size_t)j * m + j], x1 = H[(size_t)(j + 1) * m + j];
-    const double d = sqrt(x0 * x0 + x1 * x1);
-    if (d == 0.0) {
-        a.cs[j] = 1.0;
-        a.sn[j] = 0.0;
-    } else {
-        a.cs[j] = x0 / d;
-        a.sn[j] = x1 / d;
+    __syncthreads();
+    if (t == 0) {
+        const double hn = sqrt(wsq);
+        const int breakdown = !(hn > 1e-14 * wn0);
+        double x0 = col[0];
+        for (int i = 0; i < j; ++i) {
+            const double x1 = col[i + 1];
+            col[i] = cs[i] * x0 + sn[i] * x1;
+            x0 = -sn[i] * x0 + cs[i] * x1;
+        }
+        const double d = sqrt(x0 * x0 + hn * hn);
+        const double c = d == 0.0 ? 1.0 : x0 / d, sj = d == 0.0 ? 0.0 : hn / d;
+        a.cs[j] = c;
+        a.sn[j] = sj;
+        col[j] = d;
+        const double gj = a.g[j];
+        a.g[j + 1] = -sj * gj;
+        a.g[j] = c * gj;
+        a.scal[0] = hn;
+        a.scal[1] = fabs(sj * gj);
+        a.scal[2] = breakdown ? 1.0 : 0.0;
+        a.scal[3] = wn0;
     }
-    H[(size_t)j * m + j] = d;
-    H[(size_t)(j + 1) * m + j] = 0.0;
-    a.g[j + 1] = -a.sn[j] * a.g[j];
-    a.g[j] = a.cs[j] * a.g[j];
-    a.scal[0] = hn;
-    a.scal[1] = fabs(a.g[j + 1]);
-    a.scal[2] = breakdown ? 1.0 : 0.0;
-    a.scal[3] = wn0;
+    __syncthreads();
+    if (t <= j) H[(size_t)t * m + j] = col[t];
+    if (t == j + 1) H[(size_t)t * m + j] = 0.0;
 }
 
 __global__ void __launch_bounds__(kKThreads) multi_dot_kernel(long N, const double* __restrict__ x,
@@ -177,6 +193,44 @@ __global__ void __launch_bounds__(kKThreads) multi_dot_kernel(long N, const doub
     chunk_range(N, &e0, &e1);
     chunk_dots(e0, e1, x, Y, ld, nv, want_xx, partial);
     if (last_cta(ticket)) finish_sums(nv + want_xx, partial, out);
+}
+
+// t[u] -= sum over G vectors v0 .. of h[v] Y_v[e + u * blockDim.x], u < E: the
+// G * E loads are issued before the FMA chains
+template <int G, int E>
+__device__ __forceinline__ void axpy_group(double (&t)[E], const double* __restrict__ Y, long ld, long e, int v0,
+                                           const double* sh_h) {
+    double yv[G][E];
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int u = 0; u < E; ++u) yv[g][u] = Y[(size_t)(v0 + g) * ld + e + u * (long)blockDim.x];
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int u = 0; u < E; ++u) t[u] = fma(-sh_h[v0 + g], yv[g][u], t[u]);
+}
+// x[e + u * blockDim.x] -= sum_v h[v] Y_v there, u < E: groups of 8 vectors, the
+// remainder as one group of its exact size (a vector at a time, each load
+// waiting for the last, it cost as much as the groups: 98 us per pass over 25
+// vectors of 1.1 M against a floor of 47 us on the FP64 pipe)
+template <int E>
+__device__ __forceinline__ void axpy_items(double* __restrict__ x, const double* __restrict__ Y, long ld, long e, int nv,
+                                           const double* sh_h) {
+    double t[E];
+#pragma unroll
+    for (int u = 0; u < E; ++u) t[u] = x[e + u * (long)blockDim.x];
+    int v = 0;
+    for (; v + 8 <= nv; v += 8) axpy_group<8, E>(t, Y, ld, e, v, sh_h);
+    switch (nv - v) {
+#define REM(R) \
+    case R: axpy_group<R, E>(t, Y, ld, e, v, sh_h); break;
+        REM(1) REM(2) REM(3) REM(4) REM(5) REM(6) REM(7)
+#undef REM
+        default: break;
+    }
+#pragma unroll
+    for (int u = 0; u < E; ++u) x[e + u * (long)blockDim.x] = t[u];
 }
 
 // x -= sign * sum_v h[v] Y_v over the chunk, then (mode 1) the dots of the new
@@ -196,21 +250,10 @@ __global__ void __launch_bounds__(kKThreads) axpy_dot_kernel(long N, double* __r
     __syncthreads();
     long e0, e1;
     chunk_range(N, &e0, &e1);
-    // the basis vectors in groups of 8: the 8 loads are issued before the
-    // dependent FMA chain (same order of the sum as one vector at a time)
-    constexpr int kAxpyGroup = 8;
-    for (long e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-        double t = x[e];
-        int v = 0;
-        for (; v + kAxpyGroup <= nv; v += kAxpyGroup) {
-            double yv[kAxpyGroup];
-#pragma unroll
-            for (int g = 0; g < kAxpyGroup; ++g) yv[g] = Y[(size_t)(v + g) * ld + e];
-#pragma unroll
-            for (int g = 0; g < kAxpyGroup; ++g) t = fma(-sh_h[v + g], yv[g], t);
-        }
-        for (; v < nv; ++v) t = fma(-sh_h[v], Y[(size_t)v * ld + e], t);
-        x[e] = t;
+    // two elements per thread at a time, one where the chunk ends
+    for (long e = e0 + threadIdx.x; e < e1; e += 2 * (long)blockDim.x) {
+        if (e + (long)blockDim.x < e1) axpy_items<2>(x, Y, ld, e, nv, sh_h);
+        else axpy_items<1>(x, Y, ld, e, nv, sh_h);
     }
     if (mode == 0) return;
     __syncthreads();
@@ -218,24 +261,17 @@ __global__ void __launch_bounds__(kKThreads) axpy_dot_kernel(long N, double* __r
     else chunk_dots(e0, e1, x, Y, ld, 0, 1, partial);
     if (last_cta(ticket)) {
         finish_sums(mode == 1 ? nv : 1, partial, out);
+        __syncthreads();
         if (mode == 3) {
             // one projection is enough unless it removed nearly all of w
             // (||w1|| < eta ||w||, eta = 0.01); otherwise the step projects
             // again (the conditional passes) and its Givens update waits for it
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                const double w1 = __ldcg(out), w0 = __ldcg(ga.h1 + ga.j + 1);
-                const unsigned need = !(w1 >= kReorthRatio * w0);
-                *reorth = need;
-                if (!need) {
-                    double* h2 = const_cast<double*>(ga.h2);
-                    for (int i = 0; i <= ga.j; ++i) h2[i] = 0.0;
-                    givens_update(ga, w1);
-                }
-            }
+            const double w1 = __ldcg(out), w0 = __ldcg(ga.h1 + ga.j + 1);
+            const unsigned need = !(w1 >= kReorthRatio * w0);
+            if (threadIdx.x == 0) *reorth = need;
+            if (!need) givens_update(ga, w1, false);
         } else if (do_givens) {
-            __syncthreads();
-            if (threadIdx.x == 0) givens_update(ga, __ldcg(out));
+            givens_update(ga, __ldcg(out), true);
         }
     }
 }
@@ -255,14 +291,22 @@ int launch_axpy_dot(long N, double* x, const double* Y, long ld, int nv, const d
     return launched(1);
 }
 
-// y = H(0:k, 0:k)^{-1} g(0:k), upper triangular
+// y = H(0:k, 0:k)^{-1} g(0:k), upper triangular (k <= 64): one warp, a row's
+// products spread over the lanes
 __global__ void solve_upper_kernel(int k, int m, const double* __restrict__ H, const double* __restrict__ g,
                                    double* __restrict__ y) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double ys[kMaxRestart];
+    const int lane = threadIdx.x;
+    if (lane >= 32 || blockIdx.x != 0) return;
     for (int i = k - 1; i >= 0; --i) {
-        double s = g[i];
-        for (int c = i + 1; c < k; ++c) s -= H[(size_t)i * m + c] * y[c];
-        y[i] = s / H[(size_t)i * m + i];
+        double s = 0.0;
+        for (int c = i + 1 + lane; c < k; c += 32) s += H[(size_t)i * m + c] * ys[c];
+        s = warp_sum(s);
+        if (lane == 0) {
+            ys[i] = (g[i] - s) / H[(size_t)i * m + i];
+            y[i] = ys[i];
+        }
+        __syncwarp();
     }
 }
 
