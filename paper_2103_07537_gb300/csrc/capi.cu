@@ -316,6 +316,7 @@ struct bamg_ctx {
            *wsq = nullptr, *H = nullptr, *cs = nullptr, *sn = nullptr, *g = nullptr, *y = nullptr,
            *scal = nullptr;
     unsigned* ticket = nullptr;  // last-CTA counter of the chunked reductions
+    cudaEvent_t step_ev = nullptr;  // the outcome of an Arnoldi step is in h_scal
     double* h_scal = nullptr;  // pinned [4]
     // host wall time of the setup phases (ms): pattern, aggregate, rap, colour, inverse, coarse, vectors,
     // learned weights
@@ -357,6 +358,7 @@ struct bamg_ctx {
         if (coarse_ev) cudaEventDestroy(coarse_ev);
         if (cap_stream) cudaStreamSynchronize(cap_stream);  // no copy into memory freed below
         if (vals_ev) cudaEventDestroy(vals_ev);
+        if (step_ev) cudaEventDestroy(step_ev);
         if (graph_exec) cudaGraphExecDestroy(graph_exec);
         if (graph) cudaGraphDestroy(graph);
         if (prof_exec) cudaGraphExecDestroy(prof_exec);
@@ -2733,14 +2735,20 @@ static int apply_profiled(bamg_ctx* h, const double* r, double* z, cudaStream_t 
     return BAMG_OK;
 }
 
-static int apply_impl(bamg_ctx* h, const double* r, double* z, cudaStream_t s) {
+// an FP32 cycle replayed from its graph, whose cast of the input may be done by
+// the kernel that writes it (apply_impl's r32_ready)
+static bool graph_cycle32(const bamg_ctx* h) {
+    return h->p.cycle_prec == 32 && h->p.use_graph && !h->prof && !h->tail_grid;
+}
+
+static int apply_impl(bamg_ctx* h, const double* r, double* z, cudaStream_t s, bool r32_ready = false) {
     if (h->prof && h->p.use_graph) return apply_profiled(h, r, z, s);
     // (a cycle with the cooperative grid tail is one launch plus casts: direct)
     if (!h->p.use_graph || h->prof || h->tail_grid) return cycle_direct(h, r, z, s);
     TRY(ensure_graph(h));
     const long N = (long)h->lev[0].n * h->b;
     if (h->p.cycle_prec == 32) {
-        TRY(launch_cast_d2f(N, r, h->r32, s));
+        if (!r32_ready) TRY(launch_cast_d2f(N, r, h->r32, s));
         BAMG_CUDA_TRY(cudaGraphLaunch(h->graph_exec, s));
         note_launch((int)h->graph_kernels);
         return launch_cast_f2d(N, h->z32, z, s);
@@ -2805,6 +2813,7 @@ static int ensure_krylov(bamg_ctx* h, int m) {
     TRY(h->alloc(&h->scal, 4));
     TRY(h->alloc(&h->ticket, 4));
     BAMG_CUDA_TRY(cudaMemsetAsync(h->ticket, 0, 4 * sizeof(unsigned), h->stream));
+    if (!h->step_ev) BAMG_CUDA_TRY(cudaEventCreateWithFlags(&h->step_ev, cudaEventDisableTiming));
     BAMG_CUDA_TRY(cudaStreamSynchronize(h->stream));
     h->m_alloc = m;
     return BAMG_OK;
@@ -2849,6 +2858,7 @@ static int fgmres_impl(bamg_t h, const double* b, double* x, double tol, int res
     const long N = (long)L0.n * h->b;
     const int bsz = h->b;
     double* hs = h->h_scal;
+    float* r32 = graph_cycle32(h) ? h->r32 : nullptr;  // the cycle's input, written with v_j
     TRY(norm_sq(h, N, b, h->wsq, s));
     BAMG_CUDA_TRY(cudaMemcpyAsync(hs, h->wsq, sizeof(double), cudaMemcpyDeviceToHost, s));
     BAMG_CUDA_TRY(cudaStreamSynchronize(s));
@@ -2879,16 +2889,19 @@ static int fgmres_impl(bamg_t h, const double* b, double* x, double tol, int res
         }
         if (total >= max_iter) break;
         PL(BAMG_K_KRYLOV, 0.0, 0.0, launch_init_g(m, h->wsq, h->g, h->scal, s));
-        PL(BAMG_K_KRYLOV, 2.0 * vN, N, launch_scale(N, h->w, h->scal, h->V, 0, s));  // v_0 = r / beta
+        PL(BAMG_K_KRYLOV, 2.0 * vN, N, launch_scale(N, h->w, h->scal, h->V, r32, 0, s));  // v_0 = r / beta
         int k = 0;
+        bool have_z = false;  // z_j is in work already
+        double res0 = beta, res1 = beta;  // the estimates of the last two steps
         for (int j = 0; j < m; ++j) {
             const double* vj = h->V + (size_t)j * N;
+            double* vn = h->V + (size_t)(j + 1) * N;
             double* zj = h->Z + (size_t)j * N;
-            TRY(apply_impl(h, vj, zj, s));
+            if (!have_z) TRY(apply_impl(h, vj, zj, s, r32 != nullptr));
             PL(BAMG_K_SPMV, spmv_bytes, spmv_flops,
                outer_spmv(h, zj, nullptr, h->w, s));
             const double nv = j + 1;
-            GivensArgs ga{j, m, h->h1, h->h2, h->H, h->cs, h->sn, h->g, h->scal};
+            GivensArgs ga{j, m, h->h1, h->h2, h->H, h->cs, h->sn, h->g, h->scal, hs, h->d_err};
             PL(BAMG_K_KRYLOV, (nv + 1) * vN, 2.0 * N * (nv + 1),
                launch_multi_dot(N, h->w, h->V, N, j + 1, 1, h->partial, h->h1, h->ticket, s));
             if (h->p.ortho == 1) {
@@ -2902,32 +2915,46 @@ static int fgmres_impl(bamg_t h, const double* b, double* x, double tol, int res
                 // classical Gram-Schmidt, projected a second time only where the
                 // norm of w left after the first projection is below 0.01 of the
                 // norm before it (the selective test of Daniel, Gragg, Kaufman and
-                // Stewart): w -= V h1 and ||w||^2 with the test; then, only if
-                // set, h2 = V^T w and w -= V h2, ||w||^2 (Givens with h1 + h2)
-                unsigned* reorth = h->ticket + 2;
+                // Stewart): w -= V h1 and ||w||^2 with the test
                 PL(BAMG_K_KRYLOV, (nv + 2) * vN, 2.0 * N * (nv + 1),
-                   launch_axpy_dot(N, h->w, h->V, N, j + 1, h->h1, 1.0, 3, h->partial, h->wsq, h->ticket, &ga, s,
-                                   nullptr, reorth));
-                PL(BAMG_K_KRYLOV, 0.0, 0.0,
-                   launch_multi_dot(N, h->w, h->V, N, j + 1, 0, h->partial, h->h2, h->ticket, s, reorth));
-                PL(BAMG_K_KRYLOV, 0.0, 0.0,
-                   launch_axpy_dot(N, h->w, h->V, N, j + 1, h->h2, 1.0, 2, h->partial, h->wsq, h->ticket, &ga, s,
-                                   reorth));
+                   launch_axpy_dot(N, h->w, h->V, N, j + 1, h->h1, 1.0, 3, h->partial, h->wsq, h->ticket, &ga, s));
             }
-            PL(BAMG_K_KRYLOV, 2.0 * vN, N, launch_scale(N, h->w, h->scal, h->V + (size_t)(j + 1) * N, 1, s));
             total++;
             h->arnoldi_steps++;
             k = j + 1;
-            BAMG_CUDA_TRY(cudaMemcpyAsync(hs, h->scal, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
+            for (bool second = false;; second = true) {
+                // The host waits for the Givens update alone.  Behind it, v_{j+1}
+                // and the next step's V-cycle are enqueued already, so that the
+                // GPU does not idle while the host reads the outcome.  None is
+                // started where the last reduction, repeated, ends the solve: the
+                // cycle behind the last step is not used.
+                BAMG_CUDA_TRY(cudaEventRecord(h->step_ev, s));
+                PL(BAMG_K_KRYLOV, 2.0 * vN, N, launch_scale(N, h->w, h->scal, vn, r32, 1, s));
+                have_z = !h->prof && j + 1 < m && total < max_iter && res1 * (res1 / res0) > tol * bnorm;
+                if (have_z) TRY(apply_impl(h, vn, zj + N, s, r32 != nullptr));
+                BAMG_CUDA_TRY(cudaEventSynchronize(h->step_ev));
+                if (second || h->p.ortho == 1 || hs[2] == 0.0) break;
+                // the second projection: h2 = V^T w and w -= V h2, ||w||^2 (Givens
+                // with h1 + h2); v_{j+1} and its cycle again
+                h->second_projections++;
+                PL(BAMG_K_KRYLOV, (nv + 1) * vN, 2.0 * N * nv,
+                   launch_multi_dot(N, h->w, h->V, N, j + 1, 0, h->partial, h->h2, h->ticket, s));
+                PL(BAMG_K_KRYLOV, (nv + 2) * vN, 2.0 * N * (nv + 1),
+                   launch_axpy_dot(N, h->w, h->V, N, j + 1, h->h2, 1.0, 2, h->partial, h->wsq, h->ticket, &ga, s));
+            }
+            if (h->p.ortho == 1) h->second_projections++;
             // a bounded wait of the cycle (grid barrier, sweep tile) that ran out
-            BAMG_CUDA_TRY(cudaMemcpyAsync(h->h_pin, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
-            if (h->p.ortho != 1)  // whether this step projected twice (statistics)
-                BAMG_CUDA_TRY(cudaMemcpyAsync(h->h_pin + 5, h->ticket + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
-            BAMG_CUDA_TRY(cudaStreamSynchronize(s));
-            if (h->h_pin[0] != 0) return map_dev_error(h->h_pin[0]);
-            h->second_projections += h->p.ortho == 1 ? 1 : (h->h_pin[5] != 0 ? 1 : 0);
-            if (!isfinite(hs[1])) return BAMG_ENAN;
-            if (hs[1] / bnorm <= tol || hs[2] != 0.0 || total >= max_iter) break;
+            if (hs[3] != 0.0) {
+                BAMG_CUDA_TRY(cudaStreamSynchronize(s));
+                return map_dev_error((int)hs[3]);
+            }
+            if (!isfinite(hs[0])) {
+                BAMG_CUDA_TRY(cudaStreamSynchronize(s));
+                return BAMG_ENAN;
+            }
+            if (hs[0] / bnorm <= tol || hs[1] != 0.0 || total >= max_iter) break;
+            res0 = res1;
+            res1 = hs[0];
         }
         PL(BAMG_K_KRYLOV, 0.0, 0.0, launch_solve_upper(k, m, h->H, h->g, h->y, s));
         PL(BAMG_K_KRYLOV, (k + 2.0) * vN, 2.0 * N * k,

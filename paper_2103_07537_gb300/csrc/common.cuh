@@ -709,19 +709,21 @@ struct GivensArgs {
     double* sn;
     double* g;
     double* scal;      // {h_{j+1,j}, |g_{j+1}|, breakdown, ||w|| before}
+    // pinned host memory: {|g_{j+1}|, breakdown, a second projection is due, *err}
+    double* host;
+    const int* err;
 };
 // out[v] = x . Y_v (v < nv) and, if want_xx, out[nv] = x . x; deterministic chunked sums
-// (cond: run only where *cond is nonzero; null = always)
 int launch_multi_dot(long N, const double* x, const double* Y, long ld, int nv, int want_xx, double* partial,
-                     double* out, unsigned* ticket, cudaStream_t s, const unsigned* cond = nullptr);
-// x -= sign * sum_v h[v] Y_v; then mode 1: out[v] = x . Y_v, mode 2: out[0] = x . x (+ Givens if ga),
-// mode 3: as 2, and *reorth = 1 when ||x||^2 < 0.5 * ga.h1[j+1] (a second projection is due; its
-// passes carry cond = reorth), else *reorth = 0, h2 = 0 and the Givens update; mode 0: nothing
+                     double* out, unsigned* ticket, cudaStream_t s);
+// x -= sign * sum_v h[v] Y_v; then mode 1: out[v] = x . Y_v, mode 2: out[0] = x . x (+ Givens with h1 + h2 if ga),
+// mode 3: as 2, and where ||x||^2 fell below 1e-4 of ga.h1[j+1] only ga.host[2] = 1 (a second projection is due),
+// else the Givens update with h1; mode 0: nothing
 int launch_axpy_dot(long N, double* x, const double* Y, long ld, int nv, const double* h, double sign, int mode,
-                    double* partial, double* out, unsigned* ticket, const GivensArgs* ga, cudaStream_t s,
-                    const unsigned* cond = nullptr, unsigned* reorth = nullptr);
+                    double* partial, double* out, unsigned* ticket, const GivensArgs* ga, cudaStream_t s);
 int launch_solve_upper(int k, int m, const double* H, const double* g, double* y, cudaStream_t s);
-int launch_scale(long N, const double* x, const double* scal, double* y, int check_breakdown, cudaStream_t s);
+int launch_scale(long N, const double* x, const double* scal, double* y, float* y32, int check_breakdown,
+                 cudaStream_t s);
 int launch_init_g(int m, const double* bsq, double* g, double* scal, cudaStream_t s);
 
 }  // namespace bamg

@@ -177,6 +177,12 @@ __device__ void givens_update(const GivensArgs& a, double wsq, bool with_h2) {
         a.scal[1] = fabs(sj * gj);
         a.scal[2] = breakdown ? 1.0 : 0.0;
         a.scal[3] = wn0;
+        // the step's outcome for the host, which waits for this kernel only
+        a.host[0] = fabs(sj * gj);
+        a.host[1] = breakdown ? 1.0 : 0.0;
+        a.host[2] = 0.0;
+        a.host[3] = (double)__ldcg(a.err);
+        __threadfence_system();
     }
     __syncthreads();
     if (t <= j) H[(size_t)t * m + j] = col[t];
@@ -186,9 +192,7 @@ __device__ void givens_update(const GivensArgs& a, double wsq, bool with_h2) {
 __global__ void __launch_bounds__(kKThreads) multi_dot_kernel(long N, const double* __restrict__ x,
                                                               const double* __restrict__ Y, long ld, int nv,
                                                               int want_xx, double* __restrict__ partial,
-                                                              double* __restrict__ out, unsigned* ticket,
-                                                              const unsigned* cond) {
-    if (cond && __ldcg(cond) == 0u) return;  // a conditional pass that is not needed (every CTA)
+                                                              double* __restrict__ out, unsigned* ticket) {
     long e0, e1;
     chunk_range(N, &e0, &e1);
     chunk_dots(e0, e1, x, Y, ld, nv, want_xx, partial);
@@ -236,15 +240,12 @@ __device__ __forceinline__ void axpy_items(double* __restrict__ x, const double*
 // x -= sign * sum_v h[v] Y_v over the chunk, then (mode 1) the dots of the new
 // x with Y_0..Y_{nv-1} into out, (mode 2) its squared norm into out (and the
 // Givens update when do_givens), (mode 3) as 2, with the reorthogonalisation
-// test of the Arnoldi step in the last CTA, (mode 0) nothing.  cond: the pass
-// runs only where *cond is nonzero.
+// test of the Arnoldi step in the last CTA, (mode 0) nothing.
 __global__ void __launch_bounds__(kKThreads) axpy_dot_kernel(long N, double* __restrict__ x,
                                                              const double* __restrict__ Y, long ld, int nv,
                                                              const double* __restrict__ h, double sign, int mode,
                                                              double* __restrict__ partial, double* __restrict__ out,
-                                                             unsigned* ticket, GivensArgs ga, int do_givens,
-                                                             const unsigned* cond, unsigned* reorth) {
-    if (cond && __ldcg(cond) == 0u) return;
+                                                             unsigned* ticket, GivensArgs ga, int do_givens) {
     __shared__ double sh_h[kMaxRestart + 1];
     for (int v = threadIdx.x; v < nv; v += blockDim.x) sh_h[v] = sign * h[v];
     __syncthreads();
@@ -268,8 +269,12 @@ __global__ void __launch_bounds__(kKThreads) axpy_dot_kernel(long N, double* __r
             // again (the conditional passes) and its Givens update waits for it
             const double w1 = __ldcg(out), w0 = __ldcg(ga.h1 + ga.j + 1);
             const unsigned need = !(w1 >= kReorthRatio * w0);
-            if (threadIdx.x == 0) *reorth = need;
             if (!need) givens_update(ga, w1, false);
+            else if (threadIdx.x == 0) {
+                ga.host[2] = 1.0;
+                ga.host[3] = (double)__ldcg(ga.err);
+                __threadfence_system();
+            }
         } else if (do_givens) {
             givens_update(ga, __ldcg(out), true);
         }
@@ -277,17 +282,16 @@ __global__ void __launch_bounds__(kKThreads) axpy_dot_kernel(long N, double* __r
 }
 
 int launch_multi_dot(long N, const double* x, const double* Y, long ld, int nv, int want_xx, double* partial,
-                     double* out, unsigned* ticket, cudaStream_t s, const unsigned* cond) {
-    multi_dot_kernel<<<krylov_chunks(N), kKThreads, 0, s>>>(N, x, Y, ld, nv, want_xx, partial, out, ticket, cond);
+                     double* out, unsigned* ticket, cudaStream_t s) {
+    multi_dot_kernel<<<krylov_chunks(N), kKThreads, 0, s>>>(N, x, Y, ld, nv, want_xx, partial, out, ticket);
     return launched(1);
 }
 int launch_axpy_dot(long N, double* x, const double* Y, long ld, int nv, const double* h, double sign, int mode,
-                    double* partial, double* out, unsigned* ticket, const GivensArgs* ga, cudaStream_t s,
-                    const unsigned* cond, unsigned* reorth) {
+                    double* partial, double* out, unsigned* ticket, const GivensArgs* ga, cudaStream_t s) {
     GivensArgs g{};
     if (ga) g = *ga;
     axpy_dot_kernel<<<krylov_chunks(N), kKThreads, 0, s>>>(N, x, Y, ld, nv, h, sign, mode, partial, out, ticket, g,
-                                                           ga ? 1 : 0, cond, reorth);
+                                                           ga ? 1 : 0);
     return launched(1);
 }
 
@@ -310,16 +314,20 @@ __global__ void solve_upper_kernel(int k, int m, const double* __restrict__ H, c
     }
 }
 
-// y = x / scal[0] unless the breakdown flag scal[2] is set
+// y = x / scal[0] unless the breakdown flag scal[2] is set; y32 (optional): the
+// same rounded to FP32, the input of an FP32 cycle (its cast pass saved)
 __global__ void scale_kernel(long N, const double* __restrict__ x, const double* __restrict__ scal,
-                             double* __restrict__ y, int check_breakdown) {
+                             double* __restrict__ y, float* __restrict__ y32, int check_breakdown) {
     if (check_breakdown && scal[2] != 0.0) return;
     // one division per thread and a product per element: an FP64 division
     // per element costs about ten FP64 operations, and GB300 issues two per
     // clock per SM (within an ulp of the quotient)
     const double rden = 1.0 / scal[0];
-    for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < N; e += (long)gridDim.x * blockDim.x)
-        y[e] = x[e] * rden;
+    for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < N; e += (long)gridDim.x * blockDim.x) {
+        const double v = x[e] * rden;
+        y[e] = v;
+        if (y32) y32[e] = (float)v;
+    }
 }
 
 // g = (beta, 0, ..., 0) with beta = sqrt(*bsq); scal[0] = beta
@@ -335,9 +343,10 @@ int launch_solve_upper(int k, int m, const double* H, const double* g, double* y
     solve_upper_kernel<<<1, 32, 0, s>>>(k, m, H, g, y);
     return launched(1);
 }
-int launch_scale(long N, const double* x, const double* scal, double* y, int check_breakdown, cudaStream_t s) {
+int launch_scale(long N, const double* x, const double* scal, double* y, float* y32, int check_breakdown,
+                 cudaStream_t s) {
     long g = (N + 255) / 256;
-    scale_kernel<<<(int)(g < 1216 ? (g > 0 ? g : 1) : 1216), 256, 0, s>>>(N, x, scal, y, check_breakdown);
+    scale_kernel<<<(int)(g < 1216 ? (g > 0 ? g : 1) : 1216), 256, 0, s>>>(N, x, scal, y, y32, check_breakdown);
     return launched(1);
 }
 int launch_init_g(int m, const double* bsq, double* g, double* scal, cudaStream_t s) {
