@@ -985,8 +985,8 @@ static int autotune_levels(bamg_ctx* h, cudaStream_t s) {
         // Levels whose values exceed L2 are timed over every colour of the
         // field step (the average per launch): one colour launched again and
         // again would be read from L2, which the cycle's colours never are.
-        // (3D, 64^3 cells: 12.6 us against 15 us per launch in the cycle, and
-        // another mapping in front.)
+        // (3D, 64^3 cells, FP32, thread per row: the first colour alone 12.4 us,
+        // the average over the step 18.0 us.)
         int l2 = 0, dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
@@ -1050,10 +1050,8 @@ static int autotune_levels(bamg_ctx* h, cudaStream_t s) {
             // zero and a step from an iterate, every colour of field 0, in
             // programmatic dependent launches (each kernel's loads before its
             // wait overlap the previous colour, which one colour launched
-            // alone does not show: 3D level 1, four warps per node 7% faster in
-            // the cycle and within 3% alone; 2D 128^2 level 0 FP64, four lanes
-            // per row against warp per node: cycle 207 against 221 us, alone a
-            // near tie that went either way)
+            // alone does not show, and near ties there went either way: 48
+            // systems, FP32: cycle 733 us by the first choice, 700 us by this)
             PdlScope pdl(true);
             const int c_hi = h->nf > 1 ? L.fcol[1] : L.n_colours;
             const int lead = L.bgs_tpr;
@@ -2547,8 +2545,9 @@ static int setup_tail(bamg_ctx* h, cudaStream_t s) {
 // run as one launch per cycle, from the finest such level down, in the default
 // configuration (the forced row mappings, the recorded tail and the other
 // sub-solvers keep their own launches).  Wherever they fit they are the faster
-// form: a colour step of up to 1200 nodes takes 0.9 to 1.6 us inside the cluster
-// and 2.1 to 2.5 us as a kernel.
+// form.  Whole cycles, launches against the cluster: FP32 with 1089 nodes 45 ->
+// 39 us, with 625 nodes of 6 unknowns 75 -> 51 us, FP64 with 625 nodes 109 -> 94
+// us, 2D 4-field 128^2 FP64 221 -> 207 us with the same level-0 mapping.
 static int setup_coarse_cycle(bamg_ctx* h, cudaStream_t s) {
     h->l_cc = -1;
     const amg_params& p = h->p;

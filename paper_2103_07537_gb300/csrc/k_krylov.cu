@@ -144,7 +144,7 @@ __device__ __forceinline__ void finish_sums(int nv, const double* partial, doubl
 // residual estimate |g_{j+1}|.  scal = {h_{j+1,j}, |g_{j+1}|, breakdown, ||w||
 // before orthogonalising}.  The column and the rotations are loaded and stored
 // by all threads; one thread applies them in shared memory (a chain of two FP64
-// operations per rotation; through global memory it took 15 us at step 50).
+// operations per rotation instead of round trips through L2).
 __device__ void givens_update(const GivensArgs& a, double wsq, bool with_h2) {
     __shared__ double col[kMaxRestart + 2], cs[kMaxRestart], sn[kMaxRestart];
     const int j = a.j, m = a.m, t = threadIdx.x;
@@ -215,9 +215,9 @@ __device__ __forceinline__ void axpy_group(double (&t)[E], const double* __restr
         for (int u = 0; u < E; ++u) t[u] = fma(-sh_h[v0 + g], yv[g][u], t[u]);
 }
 // x[e + u * blockDim.x] -= sum_v h[v] Y_v there, u < E: groups of 8 vectors, the
-// remainder as one group of its exact size (a vector at a time, each load
-// waiting for the last, it cost as much as the groups: 98 us per pass over 25
-// vectors of 1.1 M against a floor of 47 us on the FP64 pipe)
+// remainder as one group of its exact size (a vector at a time waits for each
+// load).  Averages over 50 steps on 1.1 M unknowns, 25 vectors a pass: 99 us,
+// this way 87 us; the FP64 pipe's floor is 49 us, HBM's 34 us
 template <int E>
 __device__ __forceinline__ void axpy_items(double* __restrict__ x, const double* __restrict__ Y, long ld, long e, int nv,
                                            const double* sh_h) {
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kKThreads) axpy_dot_kernel(long N, double* __r
         if (mode == 3) {
             // one projection is enough unless it removed nearly all of w
             // (||w1|| < eta ||w||, eta = 0.01); otherwise the step projects
-            // again (the conditional passes) and its Givens update waits for it
+            // again and its Givens update waits for that
             const double w1 = __ldcg(out), w0 = __ldcg(ga.h1 + ga.j + 1);
             const unsigned need = !(w1 >= kReorthRatio * w0);
             if (!need) givens_update(ga, w1, false);

@@ -187,11 +187,11 @@ __device__ __forceinline__ void st_relaxed(int* p, int v) {
 // Those belong to its own chunk or to chunks taken earlier by running CTAs, so
 // some node can always be decided, whatever part of the grid is resident.
 // Every wait is bounded all the same: kChunkSpins polls, then the failure word
-// is set and every CTA leaves.  (Rounds over all nodes, one launch or two per
-// round, cost 13 to 26 us for each step of the dependency chain -- 455 steps
-// for the colouring of the 65^3 grid, 128 for its aggregation -- where a step
-// here is a store and a poll, about 1 us through L2 and less inside a CTA:
-// 3D setup, 65^3 nodes: colouring 5.5 ms, aggregation 3.4 ms as rounds.)
+// is set and every CTA leaves.  Bound by the chain of dependent nodes.  (Rounds
+// over all nodes cost a launch of 12 us for each step of the colouring's chain
+// and two of 21 us together for the aggregation's, where a step here is a store
+// and a poll.  3D, 65^3 nodes and the level below: colouring 6.7 -> 2.2 ms,
+// aggregation 3.7 -> 0.9 ms; 2D, 129^2 nodes: first colouring 1.28 -> 0.80 ms.)
 constexpr int kChunk = 256;
 constexpr int kChunkCtas = 4;  // CTAs per SM (the window of nodes in work)
 constexpr int kChunkSpins = 1 << 22;  // at least half a microsecond each
@@ -617,8 +617,8 @@ int colour_nodes(int n, const int* rp, const int* ci, int* colour, int* d_flag, 
                  int* n_colours, int* d_queue) {
     // Graphs of up to kWorklistMaxNodes nodes may use 255 colours and must be
     // structurally symmetric: one that is not goes to colour_worklist_kernel,
-    // whose counts of uncoloured neighbours report it.  (That kernel, one CTA,
-    // took 1.5 ms for 129^2 nodes.)  Larger graphs may use kMaxColours.
+    // whose counts of uncoloured neighbours report it (one CTA: 1.28 ms for
+    // 129^2 nodes against 0.80 ms).  Larger graphs may use kMaxColours.
     const bool small = n <= kWorklistMaxNodes;
     BAMG_CUDA_TRY(cudaMemsetAsync(colour, 0xff, sizeof(int) * (size_t)n, s));
     BAMG_CUDA_TRY(cudaMemsetAsync(d_flag, 0, 4 * sizeof(int), s));
@@ -649,8 +649,8 @@ int colour_nodes(int n, const int* rp, const int* ci, int* colour, int* d_flag, 
 // Nodes ordered by (colour, index): a counting sort over tiles of kChunk nodes.
 // count[c * tiles + t] = nodes of colour c in tile t; their exclusive scan is
 // the first place of every (colour, tile), and a node's place follows from the
-// lower nodes of its colour in its tile.  (One stable compaction per colour,
-// six launches each, took 0.2 ms a level.)
+// lower nodes of its colour in its tile.  (One stable compaction per colour was
+// six launches each.)
 __global__ void __launch_bounds__(kChunk) colour_count_kernel(int n, int C, int tiles, const int* __restrict__ colour,
                                                               int* __restrict__ count) {
     extern __shared__ int hist[];  // C
@@ -792,7 +792,7 @@ int rap_fill_cols(int nc, const int* rp_c, const int* tmp_cols, int cap, int* ci
 // then the blocks are added one after another.  Rows of up to kRapSmem bytes
 // are accumulated in shared memory, longer ones in place: block after block
 // added to global memory is a chain of 700 round trips for a row of the 3D
-// grid (1.4 ms; 0.4 ms this way, 65^3 nodes; FP64 floor 0.19 ms).
+// grid (65^3 nodes: 1.12 ms, 0.49 ms this way; the level below 0.63, 0.14 ms).
 constexpr int kRapSmem = 8192;
 __global__ void __launch_bounds__(kRapWarps * 32)
     rap_numeric_kernel(int b, int nc, const int* __restrict__ agg_ptr, const int* __restrict__ members,
@@ -1082,8 +1082,8 @@ __device__ __forceinline__ void pivot_search(const T* a, int nd, int k, T* red_v
 // alternate between two buffers: the owner of column k + 1 may send while
 // others still read those of k, and the barrier of k + 1 comes between the
 // readers of k and the writer of k + 2.  Bound by the chain of nd steps (pivot,
-// division, barrier: about 1.2 us) and by FP64 (a product and a difference per
-// entry, two a clock per SM: one CTA alone took 1.78 ms for nd = 150).
+// division, barrier: 3.4 us each) and by FP64 (a product and a difference per
+// entry, two a clock per SM).  nd = 150: 0.51 ms, one CTA alone 1.78 ms.
 template <typename T>
 __global__ void __launch_bounds__(kClusterLuThreads) lu_cluster_kernel(int nd, T* __restrict__ g, const T* __restrict__ norm,
                                                                        int* __restrict__ piv, int* err) {
