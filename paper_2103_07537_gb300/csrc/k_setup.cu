@@ -426,7 +426,11 @@ constexpr int kMaxColours = 128;
 // First fit over chunks (see take_chunk): a thread walks the lower entries of
 // its row, notes their colours and stops at the first uncoloured one.  The
 // chunk's own colours are kept in shared memory, where most of the chain of a
-// grid's rows runs.  colour: -1 everywhere on entry; ctl: colour count, failure
+// grid's rows runs.  A warp none of whose lanes can go on polls one entry per
+// lane: the walk of four entries, repeated while waiting, cost the running warps
+// their issue slots (colouring of the 3D setup, 65^3 nodes: 2.0 ms, 1.1 ms this
+// way; of the 2D one, 129^2 nodes: 1.1 and 0.72 ms; chunks of 512 and 1024 nodes
+// are as fast).  colour: -1 everywhere on entry; ctl: colour count, failure
 // word (1: a colour of `limit` or more was needed, 2: a wait ran out), ticket.
 __global__ void __launch_bounds__(kChunk) colour_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci,
                                                         int* colour, int* ctl, int limit) {
@@ -444,8 +448,10 @@ __global__ void __launch_bounds__(kChunk) colour_kernel(int n, const int* __rest
         int k = done ? 0 : rp[i];
         const int k1 = done ? 0 : rp[i + 1];
         unsigned long long used[4] = {0ull, 0ull, 0ull, 0ull};
-        for (int spins = 0; __any_sync(0xffffffffu, !done); ++spins) {
+        int spins = 0;
+        while (__any_sync(0xffffffffu, !done)) {
             bool moved = false;
+            int wait_for = 0;  // the entry a lane stopped at
             if (!done) {
                 int j[U], c[U];
 #pragma unroll
@@ -471,6 +477,7 @@ __global__ void __launch_bounds__(kChunk) colour_kernel(int n, const int* __rest
                 }
                 k += adv;
                 moved = adv > 0 || end;
+                wait_for = j[0];
                 if (end) {  // the smallest colour not in use
                     int cc = 256;
 #pragma unroll
@@ -486,11 +493,20 @@ __global__ void __launch_bounds__(kChunk) colour_kernel(int n, const int* __rest
                     done = true;
                 }
             }
-            if (!__any_sync(0xffffffffu, moved)) {
+            if (__any_sync(0xffffffffu, moved)) continue;
+            // every lane waits: polls of one entry each until one is coloured
+            bool left = false;
+            for (;; ++spins) {
+                const int c = done ? -1 : wait_for >= base ? sc[wait_for - base] : ld_relaxed(colour + wait_for);
+                if (__any_sync(0xffffffffu, c >= 0)) break;
                 if (spins > kChunkSpins) st_relaxed(ctl + 1, 2);
-                if ((spins & 1023) == 1023 && ld_relaxed(ctl + 1) != 0) break;
+                if ((spins & 1023) == 1023 && __any_sync(0xffffffffu, ld_relaxed(ctl + 1) != 0)) {
+                    left = true;
+                    break;
+                }
                 __nanosleep(20);
             }
+            if (left) break;
         }
     }
 #pragma unroll
