@@ -2858,6 +2858,8 @@ static int fgmres_impl(bamg_t h, const double* b, double* x, double tol, int res
     const int bsz = h->b;
     double* hs = h->h_scal;
     float* r32 = graph_cycle32(h) ? h->r32 : nullptr;  // the cycle's input, written with v_j
+    unsigned* reorth = h->ticket + 2;
+    bool expect_second = false;
     TRY(norm_sq(h, N, b, h->wsq, s));
     BAMG_CUDA_TRY(cudaMemcpyAsync(hs, h->wsq, sizeof(double), cudaMemcpyDeviceToHost, s));
     BAMG_CUDA_TRY(cudaStreamSynchronize(s));
@@ -2900,7 +2902,7 @@ static int fgmres_impl(bamg_t h, const double* b, double* x, double tol, int res
             PL(BAMG_K_SPMV, spmv_bytes, spmv_flops,
                outer_spmv(h, zj, nullptr, h->w, s));
             const double nv = j + 1;
-            GivensArgs ga{j, m, h->h1, h->h2, h->H, h->cs, h->sn, h->g, h->scal, hs, h->d_err};
+            GivensArgs ga{j, m, h->h1, h->h2, h->H, h->cs, h->sn, h->g, h->scal, hs, reorth, h->d_err};
             PL(BAMG_K_KRYLOV, (nv + 1) * vN, 2.0 * N * (nv + 1),
                launch_multi_dot(N, h->w, h->V, N, j + 1, 1, h->partial, h->h1, h->ticket, s));
             if (h->p.ortho == 1) {
@@ -2921,27 +2923,39 @@ static int fgmres_impl(bamg_t h, const double* b, double* x, double tol, int res
             total++;
             h->arnoldi_steps++;
             k = j + 1;
-            for (bool second = false;; second = true) {
+            // the second projection, which runs where the test asks for it: h2 =
+            // V^T w and w -= V h2, ||w||^2 (Givens with h1 + h2)
+            auto second_projection = [&]() {
+                PL(BAMG_K_KRYLOV, (nv + 1) * vN, 2.0 * N * nv,
+                   launch_multi_dot(N, h->w, h->V, N, j + 1, 0, h->partial, h->h2, h->ticket, s, reorth));
+                PL(BAMG_K_KRYLOV, (nv + 2) * vN, 2.0 * N * (nv + 1),
+                   launch_axpy_dot(N, h->w, h->V, N, j + 1, h->h2, 1.0, 2, h->partial, h->wsq, h->ticket, &ga, s,
+                                   reorth));
+                return (int)BAMG_OK;
+            };
+            if (h->p.ortho != 1 && expect_second) TRY(second_projection());
+            for (;;) {
                 // The host waits for the Givens update alone.  Behind it, v_{j+1}
                 // and the next step's V-cycle are enqueued already, so that the
                 // GPU does not idle while the host reads the outcome.  None is
-                // started where the last reduction, repeated, ends the solve: the
-                // cycle behind the last step is not used.
+                // started in the first step and where the last reduction,
+                // repeated, ends the solve: the cycle behind the last step is
+                // not used.
                 BAMG_CUDA_TRY(cudaEventRecord(h->step_ev, s));
                 PL(BAMG_K_KRYLOV, 2.0 * vN, N, launch_scale(N, h->w, h->scal, vn, r32, 1, s));
-                have_z = !h->prof && j + 1 < m && total < max_iter && res1 * (res1 / res0) > tol * bnorm;
+                have_z = !h->prof && total > 1 && j + 1 < m && total < max_iter && res1 * (res1 / res0) > tol * bnorm;
                 if (have_z) TRY(apply_impl(h, vn, zj + N, s, r32 != nullptr));
                 BAMG_CUDA_TRY(cudaEventSynchronize(h->step_ev));
-                if (second || h->p.ortho == 1 || hs[2] == 0.0) break;
-                // the second projection: h2 = V^T w and w -= V h2, ||w||^2 (Givens
-                // with h1 + h2); v_{j+1} and its cycle again
-                h->second_projections++;
-                PL(BAMG_K_KRYLOV, (nv + 1) * vN, 2.0 * N * nv,
-                   launch_multi_dot(N, h->w, h->V, N, j + 1, 0, h->partial, h->h2, h->ticket, s));
-                PL(BAMG_K_KRYLOV, (nv + 2) * vN, 2.0 * N * (nv + 1),
-                   launch_axpy_dot(N, h->w, h->V, N, j + 1, h->h2, 1.0, 2, h->partial, h->wsq, h->ticket, &ga, s));
+                if (h->p.ortho == 1 || hs[2] == 0.0) break;
+                TRY(second_projection());  // and v_{j+1} and its cycle again
             }
+            // Solves that project twice once do so again: from then on the two
+            // passes are enqueued ahead of the wait (empty where not needed)
             if (h->p.ortho == 1) h->second_projections++;
+            else if (hs[4] != 0.0) {
+                h->second_projections++;
+                expect_second = true;
+            }
             // a bounded wait of the cycle (grid barrier, sweep tile) that ran out
             if (hs[3] != 0.0) {
                 BAMG_CUDA_TRY(cudaStreamSynchronize(s));

@@ -709,18 +709,22 @@ struct GivensArgs {
     double* sn;
     double* g;
     double* scal;      // {h_{j+1,j}, |g_{j+1}|, breakdown, ||w|| before}
-    // pinned host memory: {|g_{j+1}|, breakdown, a second projection is due, *err}
+    // pinned host memory: {|g_{j+1}|, breakdown, a second projection is due and
+    // not done, *err, a second projection was found due}
     double* host;
+    unsigned* reorth;  // the last of these for the conditional passes
     const int* err;
 };
 // out[v] = x . Y_v (v < nv) and, if want_xx, out[nv] = x . x; deterministic chunked sums
 int launch_multi_dot(long N, const double* x, const double* Y, long ld, int nv, int want_xx, double* partial,
-                     double* out, unsigned* ticket, cudaStream_t s);
+                     double* out, unsigned* ticket, cudaStream_t s, const unsigned* cond = nullptr);
 // x -= sign * sum_v h[v] Y_v; then mode 1: out[v] = x . Y_v, mode 2: out[0] = x . x (+ Givens with h1 + h2 if ga),
-// mode 3: as 2, and where ||x||^2 fell below 1e-4 of ga.h1[j+1] only ga.host[2] = 1 (a second projection is due),
-// else the Givens update with h1; mode 0: nothing
+// mode 3: as 2, and where ||x||^2 fell below 1e-4 of ga.h1[j+1] only *ga.reorth = 1 and ga.host[2] = ga.host[4] = 1
+// (a second projection is due), else the Givens update with h1; mode 0: nothing; cond: the pass runs only where
+// *cond != 0
 int launch_axpy_dot(long N, double* x, const double* Y, long ld, int nv, const double* h, double sign, int mode,
-                    double* partial, double* out, unsigned* ticket, const GivensArgs* ga, cudaStream_t s);
+                    double* partial, double* out, unsigned* ticket, const GivensArgs* ga, cudaStream_t s,
+                    const unsigned* cond = nullptr);
 int launch_solve_upper(int k, int m, const double* H, const double* g, double* y, cudaStream_t s);
 int launch_scale(long N, const double* x, const double* scal, double* y, float* y32, int check_breakdown,
                  cudaStream_t s);
