@@ -2544,11 +2544,19 @@ static int setup_tail(bamg_ctx* h, cudaStream_t s) {
 // The coarse levels whose rows and vectors fit the shared memory of one cluster
 // run as one launch per cycle, from the finest such level down, in the default
 // configuration (the forced row mappings, the recorded tail and the other
-// sub-solvers keep their own launches).  Wherever they fit they are the faster
-// form.  Whole cycles, launches against the cluster: FP32 with 1089 nodes 45 ->
-// 39 us, with 625 nodes of 6 unknowns 75 -> 51 us, FP64 with 625 nodes 109 -> 94
-// us, 2D 4-field 128^2 FP64 221 -> 207 us with the same level-0 mapping.
+// sub-solvers keep their own launches).  Sixteen SMs save the launches of a level
+// (kCcSaved us per colour step) and pay for its entries (kCcEntry us per million
+// and sweep) and for those of the coarsest inverse (kCcInverse, against a product
+// on every SM); the launch starts at the level where the sum over the levels
+// below is largest, or is not used.  The constants are fits to cycles of 2D
+// systems of 3 and 6 unknowns and 3D ones of 4, 16^2 to 128^2 and 6^3 to 24^3 cells,
+// with and without the cluster.  Launches against the cluster from level 0: FP32
+// with 289 / 1089 / 2401 / 6561 nodes of 3 unknowns 57 -> 41, 60 -> 47, 62 -> 55,
+// 68 -> 76 us, with 625 nodes of 6 unknowns 99 -> 68 us; with a coarsest system of
+// 363 / 1452 unknowns 34 -> 39, 47 -> 135 us; FP64 with 625 / 2401 nodes of 3
+// unknowns 74 -> 68, 80 -> 91 us.
 static int setup_coarse_cycle(bamg_ctx* h, cudaStream_t s) {
+    constexpr double kCcSaved[2] = {0.7, 0.45}, kCcEntry[2] = {16.0, 30.0}, kCcInverse[2] = {50.0, 25.0};  // FP32, FP64
     h->l_cc = -1;
     const amg_params& p = h->p;
     if (h->nsys != 1 || h->nf != 1 || h->nlev < 2 || h->tail_d || p.sub_solver != 0 || p.inner_sweeps > 1 ||
@@ -2577,8 +2585,9 @@ static int setup_coarse_cycle(bamg_ctx* h, cudaStream_t s) {
     h->release(bound);
     // the slices, from the coarsest level up while they fit
     CcLevel lv[kCcLevels] = {};
-    size_t smem = 0;
+    size_t smem = 0, used = 0;
     int first = last;
+    double sum = -kCcInverse[f64] * 1e-6 * (double)h->nd * (double)h->nd, best = 0.0;
     for (int l = last; l >= lo; --l) {
         CcLevel& C = lv[l - lo];
         const Level& L = h->lev[l];
@@ -2586,7 +2595,7 @@ static int setup_coarse_cycle(bamg_ctx* h, cudaStream_t s) {
         C.per = per_of(l);
         C.colours = L.n_colours;
         const size_t per = (size_t)C.per;
-        size_t at = smem;
+        size_t at = used;
         auto slot = [&](int which, size_t bytes, bool copied) {
             C.off[which] = (int)at;
             at += (bytes + (copied ? 32 : 0) + 15) / 16 * 16;
@@ -2610,8 +2619,15 @@ static int setup_coarse_cycle(bamg_ctx* h, cudaStream_t s) {
             slot(kCcAgg, per * sizeof(int), true);
         }
         if (at > (size_t)kCcMaxSmem) break;
-        smem = at;
-        first = l;
+        used = at;
+        if (l == last) continue;
+        sum += kCcSaved[f64] * C.colours * F * (p.n_pre + p.n_post) -
+               kCcEntry[f64] * 1e-6 * (double)L.nnzb * b * b * (p.n_pre + p.n_post + 1);
+        if (sum > best) {
+            best = sum;
+            first = l;
+            smem = at;
+        }
     }
     if (first >= last || !coarse_cycle_fits(b, fb, f64, ctas, smem)) return BAMG_OK;
     double bytes = 0.0, flops = 0.0;
