@@ -163,7 +163,7 @@ def reduce_timing(dist, ms, solved, device):
 # public header are part of every kernel)
 KIND_SOURCES = {
     "smooth": ["k_solve.cu", "bgs_body.cuh"], "residual": ["k_solve.cu"], "cast": ["k_solve.cu"], "coarse": ["k_solve.cu"],
-    "tail": ["k_solve.cu", "bgs_body.cuh"], "spmv": ["k_solve.cu"], "restrict": ["k_solve.cu", "k_transfer.cu"],
+    "tail": ["k_solve.cu", "k_coarse.cu", "bgs_body.cuh"], "spmv": ["k_solve.cu"], "restrict": ["k_solve.cu", "k_transfer.cu"],
     "prolong": ["k_solve.cu", "k_transfer.cu"], "krylov": ["k_krylov.cu"],
 }
 
