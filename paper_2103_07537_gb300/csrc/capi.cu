@@ -179,6 +179,9 @@ struct Level {
     double* p_v64 = nullptr;
     int *r_rp = nullptr, *r_i = nullptr, *r_q = nullptr;
     void *p_vc = nullptr, *r_vc = nullptr;  // P and R values in the cycle's storage type
+    // index tables of the coarse cycle's cluster launch (see CcLevel): functions of the level's
+    // pattern alone, built once and kept while the launch is set up again
+    int *cc_enc = nullptr, *cc_list = nullptr, *cc_off = nullptr, *cc_agg = nullptr, *cc_mem = nullptr;
 };
 
 struct ProfRec {
@@ -2631,34 +2634,46 @@ static int setup_coarse_cycle(bamg_ctx* h, cudaStream_t s) {
     }
     if (first >= last || !coarse_cycle_fits(b, fb, f64, ctas, smem)) return BAMG_OK;
     double bytes = 0.0, flops = 0.0;
+    bool launched_tables = false;
     for (int l = first; l < last; ++l) {
         CcLevel& C = lv[l - lo];
-        const Level& L = h->lev[l];
-        int *enc = nullptr, *list = nullptr, *off = nullptr, *agg = nullptr, *mem = nullptr;
-        TRY(h->alloc(&enc, (size_t)L.nnzb));
-        TRY(h->alloc(&list, (size_t)L.n));
-        TRY(h->alloc(&off, (size_t)ctas * (L.n_colours + 1)));
-        TRY(h->alloc(&agg, (size_t)L.n));
-        TRY(h->alloc(&mem, (size_t)L.n));
-        TRY(launch_cc_encode(L.nnzb, C.per, L.ci, enc, s));
-        TRY(launch_cc_list(L.n, C.per, ctas, L.n_colours, L.colour, list, off, s));
-        TRY(launch_cc_encode(L.n, lv[l + 1 - lo].per, L.agg, agg, s));
-        TRY(launch_cc_encode(L.n, C.per, L.members, mem, s));
+        Level& L = h->lev[l];
+        if (!L.cc_mem) {
+            int *enc = nullptr, *list = nullptr, *off = nullptr, *agg = nullptr, *mem = nullptr;
+            TRY(h->alloc(&enc, (size_t)L.nnzb));
+            TRY(h->alloc(&list, (size_t)L.n));
+            TRY(h->alloc(&off, (size_t)ctas * (L.n_colours + 1)));
+            TRY(h->alloc(&agg, (size_t)L.n));
+            TRY(h->alloc(&mem, (size_t)L.n));
+            TRY(launch_cc_encode(L.nnzb, C.per, L.ci, enc, s));
+            TRY(launch_cc_list(L.n, C.per, ctas, L.n_colours, L.colour, list, off, s));
+            TRY(launch_cc_encode(L.n, lv[l + 1 - lo].per, L.agg, agg, s));
+            TRY(launch_cc_encode(L.n, C.per, L.members, mem, s));
+            L.cc_enc = enc;
+            L.cc_list = list;
+            L.cc_off = off;
+            L.cc_agg = agg;
+            L.cc_mem = mem;
+            launched_tables = true;
+        }
         C.rp = L.rp;
         C.vals = f64 ? (const void*)L.vals64 : (const void*)L.vals32;
-        C.enc = enc;
+        C.enc = L.cc_enc;
         C.lowk = L.lowk;
         C.dinv = f64 ? (const void*)L.dinv64 : (const void*)L.dinv32;
         C.omega = f64 ? (const void*)L.omega_s64 : (const void*)L.omega_s32;
-        C.list = list;
-        C.list_off = off;
-        C.agg = agg;
+        C.list = L.cc_list;
+        C.list_off = L.cc_off;
+        C.agg = L.cc_agg;
         C.agg_ptr = L.agg_ptr;
-        C.members = mem;
+        C.members = L.cc_mem;
         for (int r = 0; r <= ctas; ++r) C.bound[r] = hb[(size_t)(l - lo) * bs + r];
         bytes += (double)L.nnzb * (b * b * es + 5.0) + (double)L.n * (F * fb * fb * es + 20.0);
         flops += 2.0 * L.nnzb * b * b * (p.n_pre + p.n_post + 1);
     }
+    // the cycles may run on any stream: no table is still being written when
+    // the setup (or the call that replaces the damping) returns
+    if (launched_tables) BAMG_CUDA_TRY(cudaStreamSynchronize(s));
     bytes += (double)h->nd * h->nd * (h->coarse_inv32 ? 4.0 : 8.0) + 2.0 * h->lev[first].n * b * es;
     h->cc = CcArgs{};
     h->cc.nlev = last - first + 1;
