@@ -184,18 +184,16 @@ __device__ __forceinline__ void load_row(const T* __restrict__ p, T (&out)[B]) {
     }
 }
 
-// one value, and the B values at p (alignment as load_row), read through L2
-template <typename T>
-__device__ __forceinline__ T ld_cg(const T* p) {
-    return __ldcg(p);
-}
+// The B values at p (alignment as load_row) of a vector that an earlier kernel
+// of the cycle writes: ordinary loads, for pointers without __restrict__ (see
+// pdl_wait).
 template <typename T, int B>
-__device__ __forceinline__ void load_cg(const T* p, T (&out)[B]) {
+__device__ __forceinline__ void load_vec(const T* p, T (&out)[B]) {
     constexpr int bytes_row = B * (int)sizeof(T);
     if constexpr (sizeof(T) == 4 && bytes_row % 16 == 0) {
 #pragma unroll
         for (int c = 0; c < B; c += 4) {
-            const float4 v = __ldcg(reinterpret_cast<const float4*>(p + c));
+            const float4 v = *reinterpret_cast<const float4*>(p + c);
             out[c] = v.x;
             out[c + 1] = v.y;
             out[c + 2] = v.z;
@@ -205,13 +203,56 @@ __device__ __forceinline__ void load_cg(const T* p, T (&out)[B]) {
         using V2 = typename VecOf<T>::v2;
 #pragma unroll
         for (int c = 0; c < B; c += 2) {
-            const V2 v = __ldcg(reinterpret_cast<const V2*>(p + c));
+            const V2 v = *reinterpret_cast<const V2*>(p + c);
             out[c] = v.x;
             out[c + 1] = v.y;
         }
     } else {
 #pragma unroll
-        for (int c = 0; c < B; ++c) out[c] = __ldcg(p + c);
+        for (int c = 0; c < B; ++c) out[c] = p[c];
+    }
+}
+
+// one value, and the B values at p (alignment as load_row), read through L2;
+// volatile with a memory clobber, so that the compiler keeps them behind
+// pdl_wait and behind the barriers of kernels that write and read a vector
+__device__ __forceinline__ float ld_cg(const float* p) {
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ double ld_cg(const double* p) {
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+template <typename T, int B>
+__device__ __forceinline__ void load_cg(const T* p, T (&out)[B]) {
+    constexpr int bytes_row = B * (int)sizeof(T);
+    if constexpr (sizeof(T) == 4 && bytes_row % 16 == 0) {
+#pragma unroll
+        for (int c = 0; c < B; c += 4)
+            asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(out[c]), "=f"(out[c + 1]), "=f"(out[c + 2]), "=f"(out[c + 3])
+                         : "l"(p + c)
+                         : "memory");
+    } else if constexpr (sizeof(T) == 4 && bytes_row % 8 == 0) {
+#pragma unroll
+        for (int c = 0; c < B; c += 2)
+            asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];"
+                         : "=f"(out[c]), "=f"(out[c + 1])
+                         : "l"(p + c)
+                         : "memory");
+    } else if constexpr (sizeof(T) == 8 && bytes_row % 16 == 0) {
+#pragma unroll
+        for (int c = 0; c < B; c += 2)
+            asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];"
+                         : "=d"(out[c]), "=d"(out[c + 1])
+                         : "l"(p + c)
+                         : "memory");
+    } else {
+#pragma unroll
+        for (int c = 0; c < B; ++c) out[c] = ld_cg(p + c);
     }
 }
 
@@ -236,14 +277,17 @@ inline int ceil_div(long a, long b) { return (int)((a + b - 1) / b); }
 // constant during a cycle (matrices, inverses, colour lists, dampings) may be
 // read before pdl_wait().
 //
-// Vectors that an earlier kernel writes are read through L2 (ld_cg, load_cg)
-// in these kernels, and their pointers are not const __restrict__: a CTA that
-// is resident before its predecessor has finished shares its SM's L1 with the
-// predecessor's CTAs, and a wait that returns at once (the predecessor ended
-// while the CTA loaded its matrix rows) leaves their lines there.  Measured:
-// the residual after a smoother launch read old values of x~ in the first
-// cycles of a process (cold instruction caches); through L2, or with a fence
-// after the wait, never; the L2 path costs nothing measurable.
+// What an earlier kernel writes is read, in every kernel that waits like this,
+// behind the wait and through pointers that are not __restrict__: by ordinary
+// loads (load_vec) or through L2 (ld_cg, load_cg).  The qualifier promises that
+// nothing writes the data while the kernel runs, which a predecessor still
+// draining does: it allows the read-only path, which is not coherent, and lets
+// the compiler move the loads ahead of the wait.  (With a const __restrict__
+// x~, the residual behind a smoother launch read old values in the first cycles
+// of a process; by ordinary loads, as through L2, never: 2850 first and later
+// cycles of 38 hierarchies in three processes.)  The smoother's kernels, which load their matrix rows ahead
+// of the wait, gather through L2, which measured no slower; the thread-per-row
+// product gathers through L1, whose reuse between neighbouring rows it lives on.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

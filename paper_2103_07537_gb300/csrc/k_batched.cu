@@ -360,7 +360,7 @@ int batched_lu_inverse(int nsys, int b, int max_nd, const int* node_off, const l
 template <typename T>
 __global__ void batched_gemv_kernel(int nd_total, int b, const int* __restrict__ row_sys,
                                     const int* __restrict__ node_off, const long* __restrict__ inv_off,
-                                    const double* __restrict__ inv, const T* __restrict__ x, T* __restrict__ y) {
+                                    const double* __restrict__ inv, const T* x, T* y) {
     pdl_wait();
     pdl_trigger();
     const int r = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);

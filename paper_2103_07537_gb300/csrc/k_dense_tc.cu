@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(TcGemmArgs g) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int gk = kb + kc + q;
-                ea[i][q] = (gr < g.m && gk < g.k) ? __ldcg(g.A + (size_t)gr * g.lda + gk) : 0.f;
+                ea[i][q] = (gr < g.m && gk < g.k) ? ld_cg(g.A + (size_t)gr * g.lda + gk) : 0.f;
             }
         }
 #pragma unroll
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(TcGemmArgs g) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int gk = kb + kc + q;
-                eb[i][q] = (gc < g.n && gk < g.k) ? __ldcg(g.B + (size_t)gk * g.ldb + gc) : 0.f;
+                eb[i][q] = (gc < g.n && gk < g.k) ? ld_cg(g.B + (size_t)gk * g.ldb + gc) : 0.f;
             }
         }
         // the MMAs that read this stage two slices ago are done
@@ -416,9 +416,8 @@ constexpr int kStageLd = kPanel + 1;  // padded rows of the finished-row stage
 // dynamic shared memory of the panel kernel for R rows
 constexpr size_t panel_smem(int R) { return (size_t)R * (kStageLd * sizeof(float) + 3 * sizeof(int)); }
 
-__global__ void __launch_bounds__(kPanelThreads, 1) tc_panel_kernel(int nd, int p0, float* __restrict__ a,
-                                                                    int* __restrict__ mv, int* __restrict__ perm,
-                                                                    const float* __restrict__ norm, int* err) {
+__global__ void __launch_bounds__(kPanelThreads, 1) tc_panel_kernel(int nd, int p0, float* a, int* mv, int* perm,
+                                                                    const float* norm, int* err) {
     extern __shared__ __align__(16) float pan_sh[];  // stage[R][kStageLd], where_[R], at_[R], perm_s[R]
     constexpr int NW = kPanelThreads / 32;
     // per column (double-buffered by its parity): each warp's best candidate
@@ -578,8 +577,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) tc_panel_kernel(int nd, int 
 // every source value is loaded before any store), then U12 = L11^-1 A12 on
 // the panel's rows for the columns right of the panel (L11: unit lower, the
 // panel's top nb x nb block)
-__global__ void __launch_bounds__(256) tc_swap_trsm_kernel(int nd, int p0, float* __restrict__ a,
-                                                           const int* __restrict__ mv) {
+__global__ void __launch_bounds__(256) tc_swap_trsm_kernel(int nd, int p0, float* a, const int* mv) {
     __shared__ float l11[kPanel][kPanel + 1];
     __shared__ int s_mv[3 * kPanel + 1];
     pdl_wait();
@@ -620,8 +618,7 @@ __global__ void __launch_bounds__(256) tc_swap_trsm_kernel(int nd, int p0, float
 // the inverse (forward / backward substitution on a unit vector), the block
 // and the solution columns in shared memory.  Output: dinv[(2 i + y)] as a
 // row-major kInvBlock x kInvBlock matrix, zero outside the block's size.
-__global__ void __launch_bounds__(kInvBlock) tc_diag_inv_kernel(int nd, const float* __restrict__ a,
-                                                                float* __restrict__ dinv) {
+__global__ void __launch_bounds__(kInvBlock) tc_diag_inv_kernel(int nd, const float* a, float* dinv) {
     extern __shared__ float dsh[];
     constexpr int S = kInvBlock + 1;  // padded rows
     float* blk = dsh;                  // [kInvBlock][S]
@@ -674,8 +671,7 @@ __global__ void tc_init_kernel(int nd, float* __restrict__ x, int* __restrict__ 
 
 // A^-1 = Z P: column perm[m] of the inverse is column m of Z = U^-1 L^-1;
 // pos (the position of each original row) is perm's inverse
-__global__ void tc_scatter_kernel(int nd, const float* __restrict__ z, const int* __restrict__ perm,
-                                  float* __restrict__ inv, int* __restrict__ pos) {
+__global__ void tc_scatter_kernel(int nd, const float* z, const int* perm, float* inv, int* pos) {
     pdl_wait();
     const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (long)nd * nd) return;

@@ -187,8 +187,8 @@ __global__ void __launch_bounds__(IluBlock<FB>::kThreads) ilu_fwd_kernel(BgsArgs
     const bool act = q < a.n_in_colour;
     const int f0 = a.field * FB;
     const T* __restrict__ vals = static_cast<const T*>(a.vals);
-    const T* __restrict__ x_in = static_cast<const T*>(a.x_in);
-    const T* __restrict__ uc = static_cast<const T*>(a.uc);
+    const T* x_in = static_cast<const T*>(a.x_in);
+    const T* uc = static_cast<const T*>(a.uc);
     T* xt = static_cast<T*>(a.xt);
     pdl_wait();
     pdl_trigger();
@@ -207,10 +207,10 @@ __global__ void __launch_bounds__(IluBlock<FB>::kThreads) ilu_fwd_kernel(BgsArgs
             if (x_in) {
                 T arow[B], xv[B];
                 load_row<T, B>(vb + (size_t)(k - k0) * VS, arow);
-                load_row<T, B>(x_in + (size_t)j * B, xv);
+                load_vec<T, B>(x_in + (size_t)j * B, xv);
                 if (uc) {
                     T pv[B];
-                    load_row<T, B>(uc + (size_t)__ldg(a.agg + j) * B, pv);
+                    load_vec<T, B>(uc + (size_t)__ldg(a.agg + j) * B, pv);
 #pragma unroll
                     for (int c = 0; c < B; ++c) xv[c] += pv[c];
                 }
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(IluBlock<FB>::kThreads) ilu_fwd_kernel(BgsArgs
             if (lower) {
                 T lrow[FB], yv[FB];
                 load_row<T, FB>(lu + (size_t)k * FB * FB + r * FB, lrow);
-                load_row<T, FB>(xt + (size_t)j * FB, yv);
+                load_vec<T, FB>(xt + (size_t)j * FB, yv);
 #pragma unroll
                 for (int c = 0; c < FB; ++c) acc = fma(lrow[c], yv[c], acc);
             }
@@ -254,8 +254,8 @@ __global__ void __launch_bounds__(IluBlock<FB>::kThreads) ilu_bwd_kernel(BgsArgs
     const int nloc = threadIdx.x / FB, r = threadIdx.x - nloc * FB;
     const long q = (long)blockIdx.x * (NT / FB) + nloc;
     const bool act = q < a.n_in_colour;
-    const T* __restrict__ x_in = static_cast<const T*>(a.x_in);
-    const T* __restrict__ uc = static_cast<const T*>(a.uc);
+    const T* x_in = static_cast<const T*>(a.x_in);
+    const T* uc = static_cast<const T*>(a.uc);
     T* xt = static_cast<T*>(a.xt);
     pdl_wait();
     pdl_trigger();
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(IluBlock<FB>::kThreads) ilu_bwd_kernel(BgsArgs
             const int j = __ldg(a.ci + k);
             T urow[FB], xv[FB];
             load_row<T, FB>(lu + (size_t)k * FB * FB + r * FB, urow);
-            load_row<T, FB>(xt + (size_t)j * FB, xv);
+            load_vec<T, FB>(xt + (size_t)j * FB, xv);
 #pragma unroll
             for (int c = 0; c < FB; ++c) acc = fma(urow[c], xv[c], acc);
         }
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(IluBlock<FB>::kThreads) ilu_bwd_kernel(BgsArgs
     if (!act) return;
     const T xn = sh[nloc * FB + r];
     xt[(size_t)i * FB + r] = xn;
-    T* __restrict__ x_out = static_cast<T*>(a.x_out);
+    T* x_out = static_cast<T*>(a.x_out);
     const T om = a.omega_node ? static_cast<const T*>(a.omega_node)[(size_t)i * a.F + a.field] : T(a.omega);
     const int ag = (x_in && uc) ? __ldg(a.agg + i) : 0;
     for (int m = 0; m < a.F; ++m) {

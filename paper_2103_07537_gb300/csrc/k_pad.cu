@@ -18,7 +18,7 @@ namespace bamg {
 // setup that follows, so an invalid row_ptr reads nothing out of bounds here.
 __global__ void __launch_bounds__(256) pad_values_kernel(PadMap pm, int n, int nnzb, const int* __restrict__ rp,
                                                          const int* __restrict__ ci,
-                                                         const double* __restrict__ vals, double* __restrict__ vp) {
+                                                         const double* vals, double* vp) {
     const long w = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     pdl_wait();
@@ -56,7 +56,7 @@ int launch_pad_values(const PadMap& pm, int n, int nnzb, const int* rp, const in
 }
 
 // xp (n x bp) from x (n x b): zero at the dummy dofs
-__global__ void pad_vec_kernel(PadMap pm, long n, const double* __restrict__ x, double* __restrict__ xp) {
+__global__ void pad_vec_kernel(PadMap pm, long n, const double* x, double* xp) {
     const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
     if (e >= n * pm.bp) return;
@@ -67,7 +67,7 @@ __global__ void pad_vec_kernel(PadMap pm, long n, const double* __restrict__ x, 
 }
 
 // x (n x b) from xp (n x bp): the given dofs
-__global__ void unpad_vec_kernel(PadMap pm, long n, const double* __restrict__ xp, double* __restrict__ x) {
+__global__ void unpad_vec_kernel(PadMap pm, long n, const double* xp, double* x) {
     const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
     if (e >= n * pm.b) return;

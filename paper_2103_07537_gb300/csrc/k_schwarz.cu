@@ -240,9 +240,8 @@ int schwarz_setup_fill(int n_agg, int F, int b, int fb, int max_m, const int* ag
 template <typename T, int B, int FB, bool FM>
 __global__ void __launch_bounds__(256) field_residual_kernel(int n, int field, const int* __restrict__ rp,
                                                              const int* __restrict__ ci, const T* __restrict__ vals,
-                                                             const T* __restrict__ x_in, const T* __restrict__ uc,
-                                                             const int* __restrict__ agg, const T* __restrict__ rhs,
-                                                             T* __restrict__ rf) {
+                                                             const T* x_in, const T* uc,
+                                                             const int* __restrict__ agg, const T* rhs, T* rf) {
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const int i = (int)(t / FB);
     if (i >= n) return;
@@ -267,12 +266,12 @@ __global__ void __launch_bounds__(256) field_residual_kernel(int n, int field, c
                 load_row<T, B>(vb + (size_t)(min(k + u, k1 - 1) - k0) * VS, a[u]);
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u) load_row<T, B>(x_in + (size_t)j[u] * B, xv[u]);
+            for (int u = 0; u < U; ++u) load_vec<T, B>(x_in + (size_t)j[u] * B, xv[u]);
             if (uc) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     T pv[B];
-                    load_row<T, B>(uc + (size_t)__ldg(agg + j[u]) * B, pv);
+                    load_vec<T, B>(uc + (size_t)__ldg(agg + j[u]) * B, pv);
 #pragma unroll
                     for (int c = 0; c < B; ++c) xv[u][c] += pv[c];
                 }

@@ -261,7 +261,7 @@ template int launch_spmv<float>(int, int, int, int, const int*, const int*, cons
 
 template <typename T>
 __global__ void restrict_kernel(int b, int nc, const int* __restrict__ agg_ptr, const int* __restrict__ members,
-                                const T* __restrict__ res, T* __restrict__ rc) {
+                                const T* res, T* rc) {
     pdl_wait();
     pdl_trigger();
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -282,8 +282,7 @@ template int launch_restrict<float>(int, int, const int*, const int*, const floa
 
 // prolongation and correction u += P uc, P piecewise constant per dof
 template <typename T>
-__global__ void prolong_kernel(int b, int n, const int* __restrict__ agg, const T* __restrict__ uc,
-                               T* __restrict__ u) {
+__global__ void prolong_kernel(int b, int n, const int* __restrict__ agg, const T* uc, T* u) {
     pdl_wait();
     pdl_trigger();
     const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -296,8 +295,7 @@ __global__ void prolong_kernel(int b, int n, const int* __restrict__ agg, const 
 // the nodes of a range that a field step leaves alone: y = x (+ P uc), or
 // zero without x (the zero initial guess)
 template <typename T>
-__global__ void copy_prolong_kernel(int b, int n, const int* __restrict__ agg, const T* __restrict__ x,
-                                    const T* __restrict__ uc, T* __restrict__ y) {
+__global__ void copy_prolong_kernel(int b, int n, const int* __restrict__ agg, const T* x, const T* uc, T* y) {
     pdl_wait();
     pdl_trigger();
     const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -465,8 +463,7 @@ int launch_lower_flags(int n, const int* rp, const int* ci, const int* colour, u
 }
 
 template <typename T, typename S>
-__global__ void dense_gemv_kernel(int nd, const S* __restrict__ ainv, const T* __restrict__ x,
-                                  T* __restrict__ y) {
+__global__ void dense_gemv_kernel(int nd, const S* __restrict__ ainv, const T* x, T* y) {
     pdl_wait();
     pdl_trigger();
     const int row = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
@@ -502,8 +499,7 @@ template int launch_dense_gemv<double, float>(int, const float*, const double*, 
 template <typename T, int B, int FB, bool FM, int G>
 __global__ void __launch_bounds__(256) spmv_tpr_kernel(int n, const int* __restrict__ rp,
                                                        const int* __restrict__ ci, const T* __restrict__ vals,
-                                                       const T* __restrict__ x, const T* __restrict__ rhs,
-                                                       T* __restrict__ y) {
+                                                       const T* x, const T* rhs, T* y) {
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const long row = t / G;  // scalar row i * B + r
     const int sl = (int)(t - row * G);
@@ -515,9 +511,9 @@ __global__ void __launch_bounds__(256) spmv_tpr_kernel(int n, const int* __restr
     if (act) {
         const int k0 = __ldg(rp + i), k1 = __ldg(rp + i + 1);
         const int kf = k0 + sl;
-        // (the wait comes before every load but the row range: the gathers go
-        // through L1, whose reuse between the rows of neighbouring nodes is
-        // worth more here than a first block loaded ahead; see pdl_wait)
+        // (the wait comes before every load but the row range, the gathers go
+        // through L1: its reuse between the rows of neighbouring nodes is worth
+        // more here than a first block loaded ahead)
         pdl_wait();
         pdl_trigger();
 #pragma unroll 4
@@ -525,7 +521,7 @@ __global__ void __launch_bounds__(256) spmv_tpr_kernel(int n, const int* __restr
             const int j = __ldg(ci + k);
             T a[B], xv[B];
             load_row<T, B>(vrow<T, B, FB, FM>(vals, k0, k1, k, r), a);
-            load_row<T, B>(x + (size_t)j * B, xv);
+            load_vec<T, B>(x + (size_t)j * B, xv);
 #pragma unroll
             for (int c = 0; c < B; ++c) acc = fma(a[c], xv[c], acc);
         }
@@ -864,7 +860,7 @@ template int launch_bgs_colour_bsp<float>(int, int, const BgsArgs&, int, cudaStr
 // with field f increased by omega x~_i.
 template <typename T, int B, int FB, bool FM>
 __global__ void __launch_bounds__(TprBlock<FB>::kThreads)
-    gs_inner_kernel(BgsArgs a, const T* __restrict__ rf, int first, int last) {
+    gs_inner_kernel(BgsArgs a, const T* rf, int first, int last) {
     __shared__ T sh_t[TprBlock<FB>::kThreads];
     const int tloc = threadIdx.x;
     const int nloc = tloc / FB, r = tloc - nloc * FB;
@@ -905,9 +901,9 @@ __global__ void __launch_bounds__(TprBlock<FB>::kThreads)
     for (int c = 0; c < FB; ++c) xn = fma(__ldg(D + c), sh_t[nloc * FB + c], xn);
     xt[(size_t)i * FB + r] = xn;
     if (!last) return;
-    const T* __restrict__ x_in = static_cast<const T*>(a.x_in);
-    const T* __restrict__ uc = static_cast<const T*>(a.uc);
-    T* __restrict__ x_out = static_cast<T*>(a.x_out);
+    const T* x_in = static_cast<const T*>(a.x_in);
+    const T* uc = static_cast<const T*>(a.uc);
+    T* x_out = static_cast<T*>(a.x_out);
     const T om = a.omega_node ? static_cast<const T*>(a.omega_node)[(size_t)i * a.F + a.field] : T(a.omega);
     const int ag = (x_in && uc) ? __ldg(a.agg + i) : 0;
     for (int m = 0; m < a.F; ++m) {
@@ -1182,7 +1178,7 @@ template int tail_cluster_size<float>(int, int, int);
 // Y[e] = X[e], two at a time (V2 = 1) where both vectors allow it: the FP64 side
 // in 16-byte loads or stores
 template <typename X, typename Y, bool V2>
-__global__ void cast_kernel(long m, const X* __restrict__ x, Y* __restrict__ y) {
+__global__ void cast_kernel(long m, const X* x, Y* y) {
     pdl_wait();
     pdl_trigger();
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long)gridDim.x * blockDim.x;

@@ -375,7 +375,7 @@ __device__ __forceinline__ float from_storage<__nv_bfloat16>(__nv_bfloat16 v) { 
 template <typename T, typename V, int B, int FB, bool ADD>
 __global__ void __launch_bounds__(256) fdiag_spmv_kernel(int nrows, const int* __restrict__ rp,
                                                           const int* __restrict__ ci, const V* __restrict__ vals,
-                                                          const T* __restrict__ x, T* __restrict__ y) {
+                                                          const T* x, T* y) {
     constexpr int F = B / FB, PB = F * FB * FB;
     const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (long)nrows * B) return;
