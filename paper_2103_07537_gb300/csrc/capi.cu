@@ -276,7 +276,7 @@ struct bamg_ctx {
     std::vector<void*> coarse_tmp;
     std::vector<void*> allocs;
     long bytes = 0;
-    int* d_err = nullptr;   // device error flags [4]
+    int* d_err = nullptr;   // device words [4]: error flag, longest row of the level checked last
     int* h_pin = nullptr;   // pinned host ints [8]
     cudaStream_t cap_stream = nullptr;
     // cycle staging (graph input/output) and FP32 boundary buffers
@@ -457,9 +457,9 @@ extern "C" int amg_gemm_tc_f32(int m, int n, int k, const float* A, int lda, con
 }
 
 
-// read the device error flags (synchronises s)
+// read the device error flag (synchronises s); h_pin[1] receives the word beside it
 static int check_dev(bamg_ctx* h, cudaStream_t s) {
-    BAMG_CUDA_TRY(cudaMemcpyAsync(h->h_pin, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    BAMG_CUDA_TRY(cudaMemcpyAsync(h->h_pin, h->d_err, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
     BAMG_CUDA_TRY(cudaStreamSynchronize(s));
     return map_dev_error(h->h_pin[0]);
 }
@@ -824,18 +824,6 @@ static int build_sweep_plan(bamg_ctx* h, Level& L, cudaStream_t s) {
     return BAMG_OK;
 }
 
-// stored blocks in the level's longest row (the staged smoother's slots)
-static int level_max_row(bamg_ctx* h, Level& L, cudaStream_t s) {
-    int* mr = nullptr;
-    TRY(h->alloc(&mr, 1));
-    TRY(launch_row_len_max(L.n, L.rp, mr, s));
-    BAMG_CUDA_TRY(cudaMemcpyAsync(h->h_pin, mr, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BAMG_CUDA_TRY(cudaStreamSynchronize(s));
-    L.max_row = h->h_pin[0];
-    h->release(mr);
-    return BAMG_OK;
-}
-
 // the sweep arguments of colours c_lo..c_hi-1 of level L
 static SweepArgs sweep_args(bamg_ctx* h, const Level& L, int c_lo, int c_hi) {
     SweepArgs sw;
@@ -894,7 +882,8 @@ static float time_launch(cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1, int rep
 // pattern again, as in a sequence of Newton or time steps) takes the
 // recorded mappings instead of timing the launches again.  Only the choice
 // of kernels is kept, never a value.  The key holds everything the choice
-// depends on: device, sizes of the level and of every colour, block shape,
+// depends on: device, sizes of the level, of its longest row (the staged
+// mapping takes rows up to a length only) and of every colour, block shape,
 // fields, precision, value layout, launch mode and sub-solver.
 struct TuneRec {
     int bgs_tpr, spmv_tpr, sweep;
@@ -912,9 +901,9 @@ static std::string tune_key(const bamg_ctx* h, const Level& L, int l) {
     int dev = -1;
     cudaGetDevice(&dev);
     std::string k = std::to_string(dev) + "/" + std::to_string(l) + "/" + std::to_string(L.n) + "/" +
-                    std::to_string(L.nnzb) + "/" + std::to_string(h->b) + "/" + std::to_string(h->fb) + "/" +
-                    std::to_string(h->nf) + "/" + std::to_string(h->nsys) + "/" + std::to_string(h->p.cycle_prec) +
-                    "/" + std::to_string(L.fm) + "/" + std::to_string(h->p.use_pdl) + "/" +
+                    std::to_string(L.nnzb) + "/" + std::to_string(L.max_row) + "/" + std::to_string(h->b) + "/" +
+                    std::to_string(h->fb) + "/" + std::to_string(h->nf) + "/" + std::to_string(h->nsys) + "/" +
+                    std::to_string(h->p.cycle_prec) + "/" + std::to_string(L.fm) + "/" + std::to_string(h->p.use_pdl) + "/" +
                     std::to_string(h->p.sub_solver) + "/" + std::to_string(h->p.sweep) + "/" +
                     std::to_string(L.sw_tiles) + "/" +
                     std::to_string(L.omega_s64 != nullptr) + "/";
@@ -952,11 +941,9 @@ static int autotune_levels(bamg_ctx* h, cudaStream_t s) {
         }
         if (L.tune_cached) {
             // (what only the candidates not taken would need is not built)
-            if (L.bgs_tpr == 4) TRY(level_max_row(h, L, s));
             if (L.sweep) TRY(build_sweep_plan(h, L, s));
             continue;
         }
-        TRY(level_max_row(h, L, s));
         if (L.sw_tiles > 0 && h->p.sweep == 0 && h->p.autotune == 1) TRY(build_sweep_plan(h, L, s));
         const size_t nb = (size_t)L.n * b;
         BAMG_CUDA_TRY(cudaMemsetAsync(L.xa, 0, nb * sizeof(T), s));
@@ -1379,8 +1366,9 @@ static int setup_impl(bamg_ctx* h, const int* row_ptr, const int* col_idx, const
     for (int l = 0;; ++l) {
         Level& L = h->lev[l];
         TRY(h->alloc(&L.diag, (size_t)L.n));
-        TRY(launch_check_pattern(L.n, L.rp, L.ci, L.diag, h->d_err, s));
+        TRY(launch_check_pattern(L.n, L.rp, L.ci, L.diag, h->d_err, s, h->d_err + 1));
         TRY(check_dev(h, s));
+        L.max_row = h->h_pin[1];
         h->t_phase[0] += ms_since(tp);
         tp = Clock::now();
         if (h->nf > 1) {

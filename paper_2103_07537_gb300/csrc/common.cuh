@@ -418,7 +418,6 @@ int launch_gs_inner(int b, int fb, const BgsArgs& a, const T* rf, bool first, bo
 // exceed shared memory
 template <typename T>
 int launch_bgs_colour_staged(int b, int fb, const BgsArgs& a, int max_row, int* err, cudaStream_t s);
-int launch_row_len_max(int n, const int* rp, int* out, cudaStream_t s);
 
 // ---- persistent multicolour sweep (k_sweep.cu) ----
 // Every colour c_lo..c_hi-1 of one field step in one launch: the colour-
@@ -588,8 +587,10 @@ int launch_cast_f2d(long m, const float* x, double* y, cudaStream_t s);
 
 // ---- setup kernels (k_setup.cu) ----
 // diag[i] = position of the diagonal block; flag kDevBadPattern on unsorted /
-// missing diagonal / out-of-range columns
-int launch_check_pattern(int n, const int* rp, const int* ci, int* diag, int* err, cudaStream_t s);
+// missing diagonal / out-of-range columns; *max_row (optional) = stored blocks
+// in the longest row
+int launch_check_pattern(int n, const int* rp, const int* ci, int* diag, int* err, cudaStream_t s,
+                         int* max_row = nullptr);
 // aggregation; returns number of aggregates (>= 0) or a negative status.
 // agg[n] out; agg_ptr[nc+1] and members[n] allocated by the caller after the
 // count is known (second call).

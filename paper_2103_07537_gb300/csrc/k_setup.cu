@@ -128,9 +128,14 @@ __device__ __forceinline__ int find_col(const int* __restrict__ ci, int k0, int 
 // i back (structural symmetry).  diag (optional) receives the position of the
 // diagonal block.  Rows of other threads are searched only inside clamped
 // bounds, so a malformed pattern is reported without reading outside it.
+// *max_row (optional, zero on entry) takes the longest row's blocks.
 __global__ void check_pattern_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci,
-                                     int* __restrict__ diag, int* err) {
+                                     int* __restrict__ diag, int* err, int* max_row) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (max_row) {
+        const int m = __reduce_max_sync(0xffffffffu, i < n ? rp[i + 1] - rp[i] : 0);
+        if ((threadIdx.x & 31) == 0) atomicMax(max_row, m);
+    }
     if (i >= n) return;
     const int nz = rp[n];
     const int k0 = rp[i], k1 = rp[i + 1];
@@ -155,9 +160,10 @@ __global__ void check_pattern_kernel(int n, const int* __restrict__ rp, const in
     if (diag) diag[i] = d;
 }
 
-int launch_check_pattern(int n, const int* rp, const int* ci, int* diag, int* err, cudaStream_t s) {
+int launch_check_pattern(int n, const int* rp, const int* ci, int* diag, int* err, cudaStream_t s, int* max_row) {
     if (n <= 0) return BAMG_OK;
-    check_pattern_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, rp, ci, diag, err);
+    if (max_row) BAMG_CUDA_TRY(cudaMemsetAsync(max_row, 0, sizeof(int), s));
+    check_pattern_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, rp, ci, diag, err, max_row);
     return launched(1);
 }
 

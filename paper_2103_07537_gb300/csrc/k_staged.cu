@@ -248,20 +248,4 @@ int launch_bgs_colour_staged(int b, int fb, const BgsArgs& a, int max_row, int* 
 template int launch_bgs_colour_staged<double>(int, int, const BgsArgs&, int, int*, cudaStream_t);
 template int launch_bgs_colour_staged<float>(int, int, const BgsArgs&, int, int*, cudaStream_t);
 
-// the largest number of stored blocks in a row
-__global__ void row_len_max_kernel(int n, const int* __restrict__ rp, int* __restrict__ out) {
-    int m = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        m = max(m, rp[i + 1] - rp[i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
-}
-int launch_row_len_max(int n, const int* rp, int* out, cudaStream_t s) {
-    if (n <= 0) return BAMG_OK;
-    BAMG_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(int), s));
-    row_len_max_kernel<<<ceil_div(n, 256) < 1024 ? ceil_div(n, 256) : 1024, 256, 0, s>>>(n, rp, out);
-    return launched(1);
-}
-
 }  // namespace bamg
