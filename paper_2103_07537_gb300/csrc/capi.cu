@@ -940,8 +940,9 @@ static int autotune_levels(bamg_ctx* h, cudaStream_t s) {
             if (hit) L.tune_cached = 1;
         }
         if (L.tune_cached) {
-            // (what only the candidates not taken would need is not built)
-            if (L.sweep) TRY(build_sweep_plan(h, L, s));
+            // (what only the candidates not taken would need is not built; a
+            // forced sweep has its plan already)
+            if (L.sweep && !L.sw_tile_ptr_d) TRY(build_sweep_plan(h, L, s));
             continue;
         }
         if (L.sw_tiles > 0 && h->p.sweep == 0 && h->p.autotune == 1) TRY(build_sweep_plan(h, L, s));
