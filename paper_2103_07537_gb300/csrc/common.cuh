@@ -312,6 +312,25 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// The dynamic shared memory that a CTA of the kernel may use on this device,
+// with the kernel's limit raised to it (0 on failure).  The limit belongs to the
+// kernel, for every host thread: set to one call's need, a setup on another
+// thread could lower it between this thread's setting and its launch.
+template <typename K>
+inline size_t smem_limit(K* kernel) {
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, (const void*)kernel) != cudaSuccess || (size_t)most < fa.sharedSizeBytes ||
+        cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)((size_t)most - fa.sharedSizeBytes)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return (size_t)most - fa.sharedSizeBytes;
+}
+
 // counts kernel launches (defined in capi.cu); while a CUDA graph is being
 // captured on this thread the count goes to the graph instead
 void note_launch(int count = 1);

@@ -349,8 +349,7 @@ int batched_lu_inverse(int nsys, int b, int max_nd, const int* node_off, const l
     const int smem_max_nd = 156;  // nd^2 doubles <= 195 KB of shared memory
     const int use_nd = max_nd <= smem_max_nd ? max_nd : 0;
     const size_t smem = sizeof(double) * ((size_t)use_nd * use_nd + 1);
-    BAMG_CUDA_TRY(cudaFuncSetAttribute(batched_lu_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(smem < 48 * 1024 ? 48 * 1024 : smem)));
+    if (smem > smem_limit(batched_lu_inverse_kernel)) return BAMG_ECUDA;
     batched_lu_inverse_kernel<<<nsys, kBatchLuThreads, smem, s>>>(b, node_off, inv_off, rp, ci, vals, work, inv, piv,
                                                                   col, use_nd, err);
     return launched(1);

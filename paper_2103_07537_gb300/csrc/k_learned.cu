@@ -422,7 +422,8 @@ int launch_mlp_grad(const uint16_t* p16, const float* x, const float* t, const i
     const int nctas = grad_ctas(n);
     const size_t smem = sizeof(GradSmem);
     // more than 48 KB of dynamic shared memory needs the opt-in (idempotent)
-    BAMG_CUDA_TRY(cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    BAMG_CUDA_TRY(cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(GradSmem)));
     float* partial = work;
     float* partial_loss = work + (size_t)nctas * BAMG_MLP_NTRAIN;
     mlp_grad_kernel<<<nctas, kGradThreads, smem, s>>>(p16, x, t, head, n, ceil_div(n, kTileRows), partial,

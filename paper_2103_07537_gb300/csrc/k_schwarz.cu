@@ -226,7 +226,7 @@ int schwarz_setup_fill(int n_agg, int F, int b, int fb, int max_m, const int* ag
     sd_fill_kernel<<<ceil_div(n_agg, 64), 64, 0, s>>>(n_agg, agg_ptr, members, rp, ci, node_field, overlap, sd_ptr,
                                                        sd_nodes);
     const size_t smem = (size_t)max_m * max_m * sizeof(double);
-    BAMG_CUDA_TRY(cudaFuncSetAttribute(sd_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > smem_limit(sd_factor_kernel)) return BAMG_ECUDA;
     sd_factor_kernel<<<n_agg * F, 128, smem, s>>>(F, b, fb, sd_ptr, sd_nodes, agg_ptr, members, rp, ci, vals, x_off,
                                                   X, err);
     return launched(2);

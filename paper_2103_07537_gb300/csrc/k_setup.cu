@@ -1219,8 +1219,7 @@ static cudaError_t launch_cluster_lu(int nd, int C, T* a, const T* norm, int* pi
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaFuncSetAttribute(lu_cluster_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)cfg.dynamicSmemBytes);
+    cudaError_t e = cfg.dynamicSmemBytes <= smem_limit(lu_cluster_kernel<T>) ? cudaSuccess : cudaErrorInvalidValue;
     if (e == cudaSuccess && C > 8)
         e = cudaFuncSetAttribute(lu_cluster_kernel<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, lu_cluster_kernel<T>, nd, a, norm, piv, err) : e;
@@ -1966,8 +1965,7 @@ int dense_lu_inverse(int nd, T* a, int* piv, T* inv, T* lt, double* work, int* e
         if constexpr (sizeof(T) == 4) {
             constexpr int NB = 16;  // the panel's nd x (NB + 1) values: 139 KB at nd 2048
             if (can_coop && nd >= 2 * sms && (smem = panel_smem<T, NB>(nd, sms)) > 0 &&
-                cudaFuncSetAttribute(lu_panel_kernel<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem) == cudaSuccess &&
+                smem <= smem_limit(lu_panel_kernel<T, NB>) &&
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lu_panel_kernel<T, NB>, kRowsThreads, smem) ==
                     cudaSuccess &&
                 per_sm >= 1) {
@@ -1990,8 +1988,7 @@ int dense_lu_inverse(int nd, T* a, int* piv, T* inv, T* lt, double* work, int* e
         // through lt, free until the transposition: 2 * sms * nd <= nd^2)
         if (!coop_done && can_coop && nd >= 2 * sms && nd <= kRowsCols * kRowsThreads &&
             (smem = rows_smem<T>(nd, sms)) > 0 &&
-            cudaFuncSetAttribute(lu_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-                cudaSuccess &&
+            smem <= smem_limit(lu_rows_kernel<T>) &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lu_rows_kernel<T>, kRowsThreads, smem) ==
                 cudaSuccess &&
             per_sm >= 1) {
@@ -2011,8 +2008,7 @@ int dense_lu_inverse(int nd, T* a, int* piv, T* inv, T* lt, double* work, int* e
         }
         per_sm = 0;
         if (!coop_done && can_coop && (smem = coop_smem<T>(nd, sms)) > 0 &&
-            cudaFuncSetAttribute(lu_coop_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-                cudaSuccess &&
+            smem <= smem_limit(lu_coop_kernel<T>) &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lu_coop_kernel<T>, kCoopThreads, smem) ==
                 cudaSuccess &&
             per_sm >= 1) {
