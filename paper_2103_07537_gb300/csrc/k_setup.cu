@@ -192,15 +192,33 @@ __device__ __forceinline__ void st_relaxed(int* p, int v) {
 // per node, and a node waits (polling L2) for the lower nodes its rule reads.
 // Those belong to its own chunk or to chunks taken earlier by running CTAs, so
 // some node can always be decided, whatever part of the grid is resident.
-// Every wait is bounded all the same: kChunkSpins polls, then the failure word
-// is set and every CTA leaves.  Bound by the chain of dependent nodes.  (Rounds
+// Every wait is bounded all the same (WaitLimit): then the failure word is set
+// and every CTA leaves.  Bound by the chain of dependent nodes.  (Rounds
 // over all nodes cost a launch of 12 us for each step of the colouring's chain
 // and two of 21 us together for the aggregation's, where a step here is a store
 // and a poll.  3D, 65^3 nodes and the level below: colouring 6.7 -> 2.2 ms,
 // aggregation 3.7 -> 0.9 ms; 2D, 129^2 nodes: first colouring 1.28 -> 0.80 ms.)
 constexpr int kChunk = 256;
 constexpr int kChunkCtas = 4;  // CTAs per SM (the window of nodes in work)
-constexpr int kChunkSpins = 1 << 22;  // at least half a microsecond each
+
+// The bound of one wait of a warp, started anew whenever the warp gets on: by
+// the clock, since polls of shared memory and of L2 take different times and a
+// wait may last as long as the chain of all nodes in work: 608 chunks on 152
+// SMs, 0.12 s for a path numbered along itself (200001 nodes: aggregation 0.13 s,
+// colouring 0.15 s).  The clock and the failure word are looked at on every
+// 1024th poll.
+constexpr unsigned long long kChunkWaitNs = 4000000000ull;
+struct WaitLimit {
+    unsigned polls = 0;
+    unsigned long long since = 0;
+    __device__ __forceinline__ bool due() { return (++polls & 1023u) == 0; }
+    __device__ __forceinline__ bool over() {
+        unsigned long long now;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+        if (since == 0) since = now;
+        return now - since > kChunkWaitNs;
+    }
+};
 
 // the next chunk's first node, or n at the end or after a failure (whole CTA)
 __device__ __forceinline__ int take_chunk(int n, int* ticket, const int* fail) {
@@ -237,7 +255,8 @@ __global__ void __launch_bounds__(kChunk) mis2_kernel(int n, const int* __restri
         const int i0 = base + (int)threadIdx.x - lane;  // the warp's first node
         bool done = i0 + lane >= n;
         int wait = -1;  // the undecided node this lane's node was last found to wait for
-        for (int spins = 0;;) {
+        WaitLimit limit;
+        for (;;) {
             if (!done) {
                 const int own = ld_relaxed(state + i0 + lane);
                 const int other = wait >= 0 ? ld_relaxed(state + wait) : kOut;
@@ -247,11 +266,14 @@ __global__ void __launch_bounds__(kChunk) mis2_kernel(int n, const int* __restri
             if (!__any_sync(kAll, !done)) break;
             const unsigned ready = __ballot_sync(kAll, !done && wait < 0);
             if (!ready) {
-                if (++spins > kChunkSpins) st_relaxed(ctl + 1, 1);
-                if ((spins & 1023) == 1023 && __any_sync(kAll, ld_relaxed(ctl + 1) != 0)) break;
+                if (limit.due()) {
+                    if (limit.over()) st_relaxed(ctl + 1, 1);
+                    if (__any_sync(kAll, ld_relaxed(ctl + 1) != 0)) break;
+                }
                 __nanosleep(100);
                 continue;
             }
+            limit = WaitLimit();
             const int src = __ffs(ready) - 1, i = i0 + src;
             const int k0 = rp[i], k1 = rp[i + 1];
             bool root = false;
@@ -454,7 +476,6 @@ __global__ void __launch_bounds__(kChunk) colour_kernel(int n, const int* __rest
         int k = done ? 0 : rp[i];
         const int k1 = done ? 0 : rp[i + 1];
         unsigned long long used[4] = {0ull, 0ull, 0ull, 0ull};
-        int spins = 0;
         while (__any_sync(0xffffffffu, !done)) {
             bool moved = false;
             int wait_for = 0;  // the entry a lane stopped at
@@ -502,13 +523,13 @@ __global__ void __launch_bounds__(kChunk) colour_kernel(int n, const int* __rest
             if (__any_sync(0xffffffffu, moved)) continue;
             // every lane waits: polls of one entry each until one is coloured
             bool left = false;
-            for (;; ++spins) {
+            for (WaitLimit wait;;) {
                 const int c = done ? -1 : wait_for >= base ? sc[wait_for - base] : ld_relaxed(colour + wait_for);
                 if (__any_sync(0xffffffffu, c >= 0)) break;
-                if (spins > kChunkSpins) st_relaxed(ctl + 1, 2);
-                if ((spins & 1023) == 1023 && __any_sync(0xffffffffu, ld_relaxed(ctl + 1) != 0)) {
-                    left = true;
-                    break;
+                if (wait.due()) {
+                    if (wait.over()) st_relaxed(ctl + 1, 2);
+                    left = __any_sync(0xffffffffu, ld_relaxed(ctl + 1) != 0);
+                    if (left) break;
                 }
                 __nanosleep(20);
             }
