@@ -15,8 +15,8 @@ namespace bamg {
 // is one product per block with the neighbour's current entries -- one gather
 // and B products, where x_in and x~ kept apart need two gathers, the colour
 // flag and B + FB products.  The higher colours' nodes still hold x_in, and
-// the nodes of one colour do not couple, so no entry is read while its node
-// is updated.  From the zero iterate (no x_in) the lower colours' x~ alone
+// the nodes of one colour do not couple (the pattern is structurally symmetric:
+// the setup refuses others), so no entry is read while its node is updated.  From the zero iterate (no x_in) the lower colours' x~ alone
 // contribute.  arow = row f0 + r of the block; forced inline so that it stays
 // in registers.
 template <typename T, int B, int FB>

@@ -265,7 +265,7 @@ struct bamg_ctx {
         cudaStream_t stream = nullptr;
         cudaEvent_t ev = nullptr;
         int status = BAMG_OK, n_colours = 0;
-        int *flag = nullptr, *queue = nullptr, *pin = nullptr;
+        int *flag = nullptr, *pin = nullptr;
     } cjob[kMaxLevels];
     // the coarsest LU enqueued on cap_stream ahead of the smoother data of the
     // finer levels (no host synchronisation inside it); its own
@@ -1194,7 +1194,6 @@ static int colour_start(bamg_ctx* h, int l, Level& L, cudaStream_t s) {
     auto& j = h->cjob[l];
     TRY(h->alloc(&L.colour, (size_t)L.n));
     TRY(h->alloc(&j.flag, 4));
-    TRY(h->alloc(&j.queue, 2 * (size_t)L.n));
     j.pin = reinterpret_cast<int*>(pin_slot());
     if (!j.pin) return BAMG_ECUDA;
     BAMG_CUDA_TRY(cudaStreamCreateWithFlags(&j.stream, cudaStreamNonBlocking));
@@ -1212,13 +1211,13 @@ static int colour_start(bamg_ctx* h, int l, Level& L, cudaStream_t s) {
         j.thread = std::thread([jp, dev, n, rp, ci, colour]() {
             int st = cudaSetDevice(dev) == cudaSuccess ? BAMG_OK : BAMG_ECUDA;
             if (st == BAMG_OK)
-                st = colour_nodes(n, rp, ci, colour, jp->flag, jp->pin, jp->stream, &jp->n_colours, jp->queue);
+                st = colour_nodes(n, rp, ci, colour, jp->flag, jp->pin, jp->stream, &jp->n_colours);
             if (cudaEventRecord(jp->ev, jp->stream) != cudaSuccess && st == BAMG_OK) st = BAMG_ECUDA;
             jp->status = st;
         });
     } catch (...) {
         // no thread: colour on the setup stream now
-        j.status = colour_nodes(n, rp, ci, colour, j.flag, j.pin, s, &j.n_colours, j.queue);
+        j.status = colour_nodes(n, rp, ci, colour, j.flag, j.pin, s, &j.n_colours);
         if (j.status == BAMG_OK) BAMG_CUDA_TRY(cudaEventRecord(j.ev, s));
     }
     return BAMG_OK;
@@ -1235,8 +1234,7 @@ static int colour_join(bamg_ctx* h, int l, Level& L, cudaStream_t s, bool* done)
     BAMG_CUDA_TRY(cudaStreamWaitEvent(s, j.ev, 0));
     L.n_colours = j.n_colours;
     h->release(j.flag);
-    h->release(j.queue);
-    j.flag = j.queue = nullptr;
+    j.flag = nullptr;
     *done = true;
     return BAMG_OK;
 }
@@ -1502,14 +1500,12 @@ static int setup_impl(bamg_ctx* h, const int* row_ptr, const int* col_idx, const
         TRY(colour_join(h, l, L, s, &coloured));
         if (!coloured) {
             TRY(h->alloc(&L.colour, (size_t)L.n));
-            int *cflag = nullptr, *queue = nullptr;
+            int* cflag = nullptr;
             TRY(h->alloc(&cflag, 4));
-            TRY(h->alloc(&queue, 2 * (size_t)L.n));
             int *g_rp = L.rp, *g_ci = L.ci;
             if (h->nf > 1) TRY(level_field_graph(h, L, &g_rp, &g_ci, s));
-            TRY(colour_nodes(L.n, g_rp, g_ci, L.colour, cflag, h->h_pin, s, &L.n_colours, queue));
+            TRY(colour_nodes(L.n, g_rp, g_ci, L.colour, cflag, h->h_pin, s, &L.n_colours));
             h->release(cflag);
-            h->release(queue);
             if (h->nf > 1) {
                 h->release(g_rp);
                 h->release(g_ci);

@@ -625,7 +625,7 @@ int aggregate_nodes(int n, const int* rp, const int* ci, int* agg, AggWork& w, i
                     int* d_scan_tmp, long scan_tmp_bytes, cudaStream_t s);
 int build_members(int n, int nc, const int* agg, int* agg_ptr, int* members, int* d_tmp,
                   cudaStream_t s);
-// Single-CTA worklist colouring (k_setup.cu): colour[n], queues qa, qb (n ints
+// Single-CTA worklist colouring (k_setup.cu), for amg_colour_noalloc: colour[n], queues qa, qb (n ints
 // each, no initial contents needed), out[0] = colour count, out[1] = 1 on
 // failure (a colour above 254 or an inconsistent pattern).  Dynamic shared
 // memory: 5 * n + 16 bytes.
@@ -637,10 +637,9 @@ constexpr int kWorklistSmemMax = kWorklistMaxNodes * 5 + 16;  // dynamic shared 
 __global__ void __launch_bounds__(1024) colour_worklist_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci,
                                        int* __restrict__ colour, int* __restrict__ qa, int* __restrict__ qb,
                                        int* __restrict__ out, const int* __restrict__ pre_err);
-// first-fit colours of every node; d_flag: 4 device ints, h_flag: 4 pinned host
-// ints, d_queue: 2n device ints of scratch
+// first-fit colours of every node; d_flag: 4 device ints, h_flag: 4 pinned host ints
 int colour_nodes(int n, const int* rp, const int* ci, int* colour, int* d_flag, int* h_flag, cudaStream_t s,
-                 int* n_colours, int* d_queue);
+                 int* n_colours);
 // colour_ptr[C+1] and nodes sorted by (colour, index); d_tmp: colour_order_ints(n, C) ints
 long colour_order_ints(int n, int C);
 int colour_order(int n, int C, const int* colour, int* colour_ptr, int* nodes, int* d_tmp,

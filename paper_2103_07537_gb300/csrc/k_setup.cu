@@ -234,7 +234,8 @@ __device__ __forceinline__ int take_chunk(int n, int* ticket, const int* fail) {
 static int chunk_grid(int n) { return std::min(ceil_div(n, kChunk), 152 * kChunkCtas); }
 
 // Roots: node i is a root when no lower node within distance 2 is one.  A new
-// root's warp marks every higher node within distance 2 as out, so most nodes
+// root's warp marks every higher node within distance 2 as out (the graph is
+// structurally symmetric: the pattern check refuses others), so most nodes
 // are decided without any work of their own.  The others are tested by their
 // warp, a lane per row of {i} + N(i): a root among the rows' lower entries
 // takes i out, an undecided entry makes i wait (it is polled alone), else i is
@@ -541,26 +542,12 @@ __global__ void __launch_bounds__(kChunk) colour_kernel(int n, const int* __rest
     if ((threadIdx.x & 31) == 0 && cmax >= 0) atomicMax(ctl, cmax + 1);
 }
 
-// *flag = 1 where a stored block (i, j) has no counterpart (j, i); warp per row
-__global__ void asymmetric_kernel(int n, const int* __restrict__ rp, const int* __restrict__ ci, int* flag) {
-    const int i = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (i >= n) return;
-    for (int k = rp[i] + (threadIdx.x & 31); k < rp[i + 1]; k += 32) {
-        const int j = ci[k];
-        int lo = rp[j], hi = rp[j + 1];
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (ci[mid] < i) lo = mid + 1;
-            else hi = mid;
-        }
-        if (lo == rp[j + 1] || ci[lo] != i) *flag = 1;
-    }
-}
-
 // Single-CTA Jones-Plassmann for graphs that fit in shared memory: a node is
 // coloured (smallest colour unused by its lower-index neighbours) as soon as
 // its count of uncoloured lower-index neighbours reaches zero; the frontier
-// of such nodes advances one step per iteration.  Same result as colour_kernel.
+// of such nodes advances one step per iteration.  Same result as colour_kernel,
+// without its host reads: the colouring of amg_colour_noalloc (129^2 nodes: 1.28
+// ms, colour_kernel 0.72 ms).
 // The count of node j is taken from row j and decremented from the rows of
 // its lower neighbours, so the rule needs a structurally symmetric pattern.
 // A pattern that is not symmetric is reported (out[1] = 1), never coloured
@@ -655,35 +642,18 @@ __global__ void __launch_bounds__(1024) colour_worklist_kernel(int n, const int*
     }
 }
 
-// d_flag: 4 device ints, h_flag: 4 pinned host ints, d_queue: 2n ints of scratch
+// d_flag: 4 device ints, h_flag: 4 pinned host ints
 int colour_nodes(int n, const int* rp, const int* ci, int* colour, int* d_flag, int* h_flag, cudaStream_t s,
-                 int* n_colours, int* d_queue) {
-    // Graphs of up to kWorklistMaxNodes nodes may use 255 colours and must be
-    // structurally symmetric: one that is not goes to colour_worklist_kernel,
-    // whose counts of uncoloured neighbours report it (one CTA: 1.28 ms for
-    // 129^2 nodes against 0.80 ms).  Larger graphs may use kMaxColours.
-    const bool small = n <= kWorklistMaxNodes;
+                 int* n_colours) {
+    // graphs of up to kWorklistMaxNodes nodes may use 255 colours, larger ones kMaxColours
+    const int limit = n <= kWorklistMaxNodes ? 255 : kMaxColours;
     BAMG_CUDA_TRY(cudaMemsetAsync(colour, 0xff, sizeof(int) * (size_t)n, s));
     BAMG_CUDA_TRY(cudaMemsetAsync(d_flag, 0, 4 * sizeof(int), s));
-    colour_kernel<<<chunk_grid(n), kChunk, 0, s>>>(n, rp, ci, colour, d_flag, small ? 255 : kMaxColours);
-    if (small) asymmetric_kernel<<<ceil_div((long)n * 32, 256), 256, 0, s>>>(n, rp, ci, d_flag + 3);
-    note_launch(small ? 2 : 1);
-    BAMG_CUDA_TRY(cudaMemcpyAsync(h_flag, d_flag, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    colour_kernel<<<chunk_grid(n), kChunk, 0, s>>>(n, rp, ci, colour, d_flag, limit);
+    note_launch(1);
+    BAMG_CUDA_TRY(cudaMemcpyAsync(h_flag, d_flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
     BAMG_CUDA_TRY(cudaStreamSynchronize(s));
     if (h_flag[1] == 2) return BAMG_ETIMEOUT;
-    if (small && h_flag[3]) {
-        const size_t smem = (size_t)n * 5 + 16;
-        // the limit is always raised to what the largest accepted graph needs,
-        // never to this call's size: amg_colour_noalloc launches the same
-        // kernel after raising it once per device, and a lower limit set here
-        // would make its next launch on a larger graph fail
-        BAMG_CUDA_TRY(cudaFuncSetAttribute(colour_worklist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           kWorklistSmemMax));
-        colour_worklist_kernel<<<1, 1024, smem, s>>>(n, rp, ci, colour, d_queue, d_queue + n, d_flag, nullptr);
-        note_launch(1);
-        BAMG_CUDA_TRY(cudaMemcpyAsync(h_flag, d_flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-        BAMG_CUDA_TRY(cudaStreamSynchronize(s));
-    }
     if (h_flag[1]) return BAMG_EUNSUPPORTED;
     *n_colours = h_flag[0];
     return BAMG_OK;
