@@ -485,6 +485,8 @@ int amg_level_copy(bamg_t h, int level, int* row_ptr, int* col_idx, double* vals
 int amg_level_ilu(bamg_t h, int level, double* lu);
 
 /* JSON summary of the hierarchy (levels, sizes, colours, bytes) into json[cap];
+ * a level's aggregation_rounds and colouring_rounds count the launches that
+ * decided its aggregates and colours (1; 0 on the coarsest level);
  * returns the length written (without the terminating zero) or a negative status. */
 int amg_stats(bamg_t h, char* json, int cap);
 

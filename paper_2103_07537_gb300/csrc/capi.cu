@@ -3345,8 +3345,9 @@ extern "C" int amg_stats(bamg_t h, char* json, int cap) {
         if (l) o += ",";
         o += "{\"n\":" + std::to_string(L.n) + ",\"nnzb\":" + std::to_string(L.nnzb) +
              ",\"colours\":" + std::to_string(L.n_colours) + ",\"aggregates\":" + std::to_string(L.n_agg) +
-             // (one launch each: no rounds)
-             ",\"aggregation_rounds\":0,\"colouring_rounds\":0" + ",\"smoother_mapping\":\"" + (L.sweep == 2     ? "sweep-split"
+             // (launches that decided the level's aggregates and colours: one each, none on the coarsest level)
+             ",\"aggregation_rounds\":" + std::to_string(l + 1 < h->nlev ? 1 : 0) +
+             ",\"colouring_rounds\":" + std::to_string(L.n_colours > 0 ? 1 : 0) + ",\"smoother_mapping\":\"" + (L.sweep == 2     ? "sweep-split"
                                           : L.sweep        ? "sweep"
                                           : L.bgs_tpr == 7 ? "block-split8"
                                           : L.bgs_tpr == 6 ? "block-split16"
