@@ -2875,7 +2875,9 @@ static int fgmres_impl(bamg_t h, const double* b, double* x, double tol, int res
     double* hs = h->h_scal;
     float* r32 = graph_cycle32(h) ? h->r32 : nullptr;  // the cycle's input, written with v_j
     unsigned* reorth = h->ticket + 2;
-    bool expect_second = false;
+    // (one level: the cycle is the coarsest solve, so A z is v up to rounding, the
+    // first projection leaves nothing of it and every step projects twice)
+    bool expect_second = h->nlev == 1;
     TRY(norm_sq(h, N, b, h->wsq, s));
     BAMG_CUDA_TRY(cudaMemcpyAsync(hs, h->wsq, sizeof(double), cudaMemcpyDeviceToHost, s));
     BAMG_CUDA_TRY(cudaStreamSynchronize(s));
@@ -2954,12 +2956,13 @@ static int fgmres_impl(bamg_t h, const double* b, double* x, double tol, int res
                 // The host waits for the Givens update alone.  Behind it, v_{j+1}
                 // and the next step's V-cycle are enqueued already, so that the
                 // GPU does not idle while the host reads the outcome.  None is
-                // started in the first step and where the last reduction,
-                // repeated, ends the solve: the cycle behind the last step is
-                // not used.
+                // started in the first step, where the last reduction, repeated,
+                // ends the solve (the cycle behind the last step is not used)
+                // and on one level, whose solves end within a step or two.
                 BAMG_CUDA_TRY(cudaEventRecord(h->step_ev, s));
                 PL(BAMG_K_KRYLOV, 2.0 * vN, N, launch_scale(N, h->w, h->scal, vn, r32, 1, s));
-                have_z = !h->prof && total > 1 && j + 1 < m && total < max_iter && res1 * (res1 / res0) > tol * bnorm;
+                have_z = !h->prof && h->nlev > 1 && total > 1 && j + 1 < m && total < max_iter &&
+                         res1 * (res1 / res0) > tol * bnorm;
                 if (have_z) TRY(apply_impl(h, vn, zj + N, s, r32 != nullptr));
                 BAMG_CUDA_TRY(cudaEventSynchronize(h->step_ev));
                 if (h->p.ortho == 1 || hs[2] == 0.0) break;
