@@ -1042,15 +1042,19 @@ static int autotune_levels(bamg_ctx* h, cudaStream_t s) {
             // programmatic dependent launches (each kernel's loads before its
             // wait overlap the previous colour, which one colour launched
             // alone does not show, and near ties there went either way: 48
-            // systems, FP32: cycle 733 us by the first choice, 700 us by this)
+            // systems, FP32: cycle 733 us by the first choice, 700 us by this);
+            // each mapping once and five times two steps, tens of launches: the
+            // first setup of a level shape pays for them
             PdlScope pdl(true);
             const int c_hi = h->nf > 1 ? L.fcol[1] : L.n_colours;
             const int lead = L.bgs_tpr;
             int best_m = 0;
             float best_us = 1e30f;
-            for (int m : {0, 5, 3, lead}) {
-                L.bgs_tpr = m;
-                const float us = time_launch(s, e0, e1, reps, [&]() {
+            const int modes[4] = {0, 5, 3, lead};
+            const int nmodes = lead == 0 || lead == 5 || lead == 3 ? 3 : 4;
+            for (int q = 0; q < nmodes; ++q) {
+                L.bgs_tpr = modes[q];
+                const float us = time_launch(s, e0, e1, 5, [&]() {
                     for (int t = 0; t < 2; ++t)
                         for (int c = 0; c < c_hi; ++c) {
                             BgsArgs ac = a;
@@ -1065,7 +1069,7 @@ static int autotune_levels(bamg_ctx* h, cudaStream_t s) {
                 });
                 if (us < best_us) {
                     best_us = us;
-                    best_m = m;
+                    best_m = modes[q];
                 }
             }
             L.bgs_tpr = best_m;
