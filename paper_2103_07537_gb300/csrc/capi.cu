@@ -1841,6 +1841,8 @@ static int setup_common(const int* row_ptr, const int* col_idx, const double* va
         const size_t NP = (size_t)n_nodes * bp;
         st = h->alloc(&h->pad_b, NP);
         if (st == BAMG_OK) st = h->alloc(&h->pad_x, NP);
+        // (stream-ordered: in place before a call on another stream uses them)
+        if (st == BAMG_OK && cudaStreamSynchronize(s) != cudaSuccess) st = BAMG_ECUDA;
         if (st != BAMG_OK) {
             amg_destroy(h);
             *out = nullptr;
