@@ -320,7 +320,7 @@ struct bamg_ctx {
            *scal = nullptr;
     unsigned* ticket = nullptr;  // last-CTA counter of the chunked reductions
     cudaEvent_t step_ev = nullptr;  // the outcome of an Arnoldi step is in h_scal
-    double* h_scal = nullptr;  // pinned [4]
+    double* h_scal = nullptr;  // pinned [16], the first five written by the Arnoldi kernels (GivensArgs::host)
     // host wall time of the setup phases (ms): pattern, aggregate, rap, colour, inverse, coarse, vectors,
     // learned weights
     double t_phase[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -2548,7 +2548,11 @@ static int setup_tail(bamg_ctx* h, cudaStream_t s) {
 // with 289 / 1089 / 2401 / 6561 nodes of 3 unknowns 57 -> 41, 60 -> 47, 62 -> 55,
 // 68 -> 76 us, with 625 nodes of 6 unknowns 99 -> 68 us; with a coarsest system of
 // 363 / 1452 unknowns 34 -> 39, 47 -> 135 us; FP64 with 625 / 2401 nodes of 3
-// unknowns 74 -> 68, 80 -> 91 us.
+// unknowns 74 -> 68, 80 -> 91 us.  By the rule, cycles down to a few coarsest
+// nodes: FP32 with 289 to 37249 nodes of 3 unknowns 59 -> 43 to 78 -> 74 us, with
+// 169 to 16641 nodes of 6 unknowns 97 -> 62 to 125 -> 113 us; FP64 with 289 to
+// 16641 nodes of 3 unknowns 70 -> 66 to 95 -> 93 us, with 169 to 16641 nodes of 6
+// unknowns 128 -> 115 to 208 -> 207.5 us.
 static int setup_coarse_cycle(bamg_ctx* h, cudaStream_t s) {
     constexpr double kCcSaved[2] = {0.7, 0.45}, kCcEntry[2] = {16.0, 30.0}, kCcInverse[2] = {50.0, 25.0};  // FP32, FP64
     h->l_cc = -1;

@@ -12,8 +12,9 @@
 // restricted form never uses the others): X_I, own_rows x m, stored column by
 // column so that the cycle reads it coalesced.  A field step is then
 //   r_f = rhs_f - A_{f,*} x_in                (one thread per scalar row)
-//   x~_i = X_I r_f|_I for the own nodes i of every aggregate I (one warp per
-//   subdomain: gather r over the subdomain, then lanes = own rows)
+//   x~_i = X_I r_f|_I for the own nodes i of every aggregate I (one CTA per
+//   subdomain: gather r over the subdomain, then lanes = own rows, the columns
+//   split over four warps)
 //   x_f += omega x~_f
 // with no dependence between subdomains, so one launch of each per field step.
 #include "common.cuh"
